@@ -244,6 +244,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // requantises and stores this thread's share of the output tile of item (b, h, mt), count index k
         auto epilogue = [&](int k, int b, int h, int mt) -> bool {
             if (!mbar_wait_nocall(o_full, (uint32_t)k & 1u, ctl, p.status, 16)) return false;
+            __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             const int row = mt * 128 + rloc;
             constexpr int OPARTS = DH / 16;                    // threads of a row that hold 16 output columns each
@@ -310,6 +311,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 ok = false;
                 break;
             }
+            __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             // ---- this thread's quarter of the score row, TMEM -> registers, in one batch
             uint32_t v[4][16];

@@ -239,6 +239,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const unsigned id_hi = HAS_MASK && lane + 32 < p.N ? mrow[lane + 32] : 0x100u;
 
             if (!mbar_wait(&s_full[g], (uint32_t)n & 1u, ctl, p.status, 25)) break;
+            __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             uint32_t v[4][16];
 #pragma unroll
@@ -353,6 +354,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             if (lane == 0) mbar_arrive(&p_ready[g]);
             // ---- output of this item: the other groups' items fill the time the P V product takes
             if (!mbar_wait(&o_full[g], (uint32_t)n & 1u, ctl, p.status, 26)) break;
+            __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             if (warp_rows) {
                 int8_t* orow = p.out + ((size_t)b * p.N + row) * HD + h * DH;

@@ -1,6 +1,7 @@
 """Thin Python binding of the iptq C-ABI library (``include/iptq.h``).
 
-Argument marshalling only: torch is used for device memory and streams; every step of the
+Argument marshalling only, natively (``csrc/binding.cpp``) for the calls a program makes once per layer and through ctypes
+for set-up and host arithmetic: torch is used for device memory and streams; every step of the
 path runs in the library's CUDA kernels.  The binding fails loudly when ``libiptq.so`` is
 missing -- there is no CPU or eager fallback.
 """
@@ -87,16 +88,21 @@ class IptqError(RuntimeError):
 
 
 _lib = None
+_nat = None          # the native half of this binding (csrc/binding.cpp), bound to the loaded library by lib()
 _vp = C.c_void_p
 
 
 def lib():
     """Load ``libiptq.so`` (built in-tree by ``paper_2511_15369_b200.build``)."""
-    global _lib
+    global _lib, _nat
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError("libiptq.so is missing: run `python -m paper_2511_15369_b200.build` "
                               "(the library has no CPU fallback)")
+        try:
+            from . import _native
+        except ImportError as e:
+            raise ImportError("_native.so is missing or does not load: run `python -m paper_2511_15369_b200.build`") from e
         L = C.CDLL(LIB_PATH)
         L.iptq_strerror.restype = C.c_char_p
         L.iptq_strerror.argtypes = [C.c_int]
@@ -161,8 +167,20 @@ def lib():
         L.iptq_metric_term.argtypes = [C.c_double, C.c_double, C.c_double, C.c_double]
         L.iptq_op_count.argtypes = [C.c_int, C.c_int, C.c_int64, C.c_int]
         L.iptq_metric_select.argtypes = [C.POINTER(C.c_double), C.c_int]
-        _lib = L
+        L.iptq_analyze_softmax.argtypes = [_vp, C.c_int64, C.c_int, C.c_double, _vp, C.c_int, _vp, _vp, _vp]
+        L.iptq_analyze_gelu.argtypes = [_vp, C.c_int64, C.c_double, C.c_double, C.c_int, _vp, C.c_int, _vp, _vp, _vp]
+        L.iptq_analyze_layernorm.argtypes = [_vp, C.c_int64, C.c_int, _vp, _vp, _vp, _vp, _vp, C.c_double, C.c_int, _vp, C.c_int,
+                                             _vp, _vp, _vp]
+        _native.bind(L._handle, _chk)
+        _lib, _nat = L, _native
     return _lib
+
+
+def native():
+    """The native entry points (tensors in, tensors out; positional arguments only)."""
+    if _nat is None:
+        lib()
+    return _nat
 
 
 def exported_symbols():
@@ -172,7 +190,8 @@ def exported_symbols():
             "iptq_unpack_int4", "iptq_linear_workspace_bytes", "iptq_linear_plan", "iptq_linear", "iptq_linear_bits", "iptq_linear_w4_static", "iptq_gather_rows", "iptq_patchify", "iptq_attention_workspace_bytes", "iptq_attention_bias_bytes", "iptq_attention_bias_prepare", "iptq_attention_block",
             "iptq_mlp_workspace_bytes", "iptq_mlp_block", "iptq_encoder_block_workspace_bytes",
             "iptq_encoder_block", "iptq_encoder_block_profiled", "iptq_workspace_init", "iptq_check", "iptq_workspace_set_wait_limit", "iptq_selftest_wait_timeout", "iptq_strerror", "iptq_launch_count",
-            "iptq_metric_softmax", "iptq_metric_gelu", "iptq_metric_layernorm", "iptq_softplus", "iptq_sqnr_db",
+            "iptq_metric_softmax", "iptq_metric_gelu", "iptq_metric_layernorm",
+            "iptq_analyze_softmax", "iptq_analyze_gelu", "iptq_analyze_layernorm", "iptq_softplus", "iptq_sqnr_db",
             "iptq_metric_term", "iptq_op_count", "iptq_metric_select"]
 
 
@@ -276,13 +295,7 @@ class Workspace:
 # ------------------------------------------------------------------ device entry points
 
 def softmax(scores, consts: SoftmaxConsts, bias=None, out=None):
-    rows, n = scores.shape
-    if out is None:
-        out = torch.empty((rows, n), dtype=torch.uint8, device=scores.device)
-    period = bias.shape[0] if bias is not None else 1
-    _chk(lib().iptq_softmax(_dp(scores), _dp(out), rows, n, _dp(bias), period, C.byref(consts), _stream()),
-         "iptq_softmax")
-    return out
+    return (_nat or native()).softmax(scores, consts, bias, out)
 
 
 SOFTMAX_TABLE_MAX = 51200
@@ -301,10 +314,7 @@ def softmax_table(consts: SoftmaxConsts, device="cuda"):
 
 
 def gelu(x, consts: GeluConsts, out=None):
-    if out is None:
-        out = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-    _chk(lib().iptq_gelu(_dp(x), _dp(out), x.numel(), C.byref(consts), _stream()), "iptq_gelu")
-    return out
+    return (_nat or native()).gelu(x, consts, out)
 
 
 GELU_TABLE_SIZE = 65536
@@ -339,6 +349,8 @@ def gelu_table(consts: GeluConsts, device="cuda"):
 
 LAYER_SOFTMAX, LAYER_GELU, LAYER_LAYERNORM = 0, 1, 2
 METRIC_WORK_BYTES = 32768
+ANALYZE_WORK_BYTES = 65536
+ANALYZE_MAX_CANDIDATES = 4
 
 
 class MetricScratch:
@@ -397,12 +409,7 @@ def metric_select(terms):
 
 
 def layernorm(x, gamma_q, beta_q, consts: LnConsts, ptf_shift=None, out=None):
-    rows, dim = x.shape
-    if out is None:
-        out = torch.empty((rows, dim), dtype=torch.int8, device=x.device)
-    _chk(lib().iptq_layernorm(_dp(x), _dp(out), rows, dim, _dp(gamma_q), _dp(beta_q), _dp(ptf_shift),
-                              C.byref(consts), _stream()), "iptq_layernorm")
-    return out
+    return (_nat or native()).layernorm(x, gamma_q, beta_q, consts, ptf_shift, out)
 
 
 def unpack_int4(w_packed):
@@ -426,14 +433,8 @@ def linear_workspace_bytes(M, N, K, w_bits=8):
 
 def linear(x, w, bias, mult, shift, ws: Workspace, out_zp=0, residual=None, residual_rq=None, w_bits=8, out=None,
            out_bits=8):
-    M, K = x.shape
-    N = w.shape[0]
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.int8, device=x.device)
-    _chk(lib().iptq_linear_bits(_dp(x), _dp(w), w_bits, _dp(bias), _dp(mult), _dp(shift), out_zp, _dp(residual),
-                                _ref(residual_rq), _dp(out), M, N, K, out_bits, ws.ptr, ws.nbytes, _stream()),
-         "iptq_linear")
-    return out
+    return (_nat or native()).linear(x, w, w_bits, bias, mult, shift, out_zp, residual, residual_rq, out_bits, ws.ptr, ws.nbytes,
+                                     out)
 
 
 STATIC_SCRATCH_BYTES = 4 << 20
@@ -456,21 +457,12 @@ def linear_w4_static(x, w_packed, bias, mult, shift, out_zp=0, residual=None, re
 
 def gather_rows(src, index, out=None):
     """dst row i = concatenation of the src rows index[i, :] (negative -> zeros); src [n_src, C] int8, index [n_dst, parts] int32."""
-    n_dst, parts = index.shape
-    C_ = src.shape[1]
-    if out is None:
-        out = torch.empty((n_dst, parts * C_), dtype=torch.int8, device=src.device)
-    _chk(lib().iptq_gather_rows(_dp(src), _dp(out), _dp(index), n_dst, parts, C_, _stream()), "iptq_gather_rows")
-    return out
+    return (_nat or native()).gather_rows(src, index, out)
 
 
 def patchify(img, patch=16, out=None):
     """img: int8 [B, C, H, W] -> patch rows int8 [B * (H/patch) * (W/patch), C * patch * patch]."""
-    B, C_, H, W = img.shape
-    if out is None:
-        out = torch.empty((B * (H // patch) * (W // patch), C_ * patch * patch), dtype=torch.int8, device=img.device)
-    _chk(lib().iptq_patchify(_dp(img), _dp(out), B, C_, H, W, patch, _stream()), "iptq_patchify")
-    return out
+    return (_nat or native()).patchify(img, patch, out)
 
 
 def attention_workspace_bytes(B, H, N, dh):
@@ -491,13 +483,7 @@ def attention_bias_prepare(bias):
 
 def attention_block(q, k, v, sm: SoftmaxConsts, out_rq: Requant, ws: Workspace, bias=None, mask_id=None, out=None,
                     bias_t=None):
-    B, H, N, dh = q.shape
-    if out is None:
-        out = torch.empty((B, N, H * dh), dtype=torch.int8, device=q.device)
-    _chk(lib().iptq_attention_block(_dp(q), _dp(k), _dp(v), _dp(out), B, H, N, dh, _dp(bias), _dp(bias_t),
-                                    _dp(mask_id), C.byref(sm), C.byref(out_rq), ws.ptr, ws.nbytes, _stream()),
-         "iptq_attention_block")
-    return out
+    return (_nat or native()).attention_block(q, k, v, sm, out_rq, ws.ptr, ws.nbytes, bias, mask_id, out, bias_t)
 
 
 def mlp_workspace_bytes(M, D, Dh, w_bits=8):
@@ -506,14 +492,8 @@ def mlp_workspace_bytes(M, D, Dh, w_bits=8):
 
 def mlp_block(x, w1, b1, m1, s1, gelu_c: GeluConsts, ws: Workspace, w2=None, b2=None, m2=None, s2=None, out_zp=0,
               residual=None, residual_rq=None, w_bits=8, out=None):
-    M, D = x.shape
-    Dh = w1.shape[0]
-    if out is None:
-        out = torch.empty((M, D if w2 is not None else Dh), dtype=torch.int8, device=x.device)
-    _chk(lib().iptq_mlp_block(_dp(x), _dp(w1), _dp(b1), _dp(m1), _dp(s1), C.byref(gelu_c), _dp(w2), _dp(b2),
-                              _dp(m2), _dp(s2), out_zp, _dp(residual), _ref(residual_rq), _dp(out), M, D, Dh,
-                              w_bits, ws.ptr, ws.nbytes, _stream()), "iptq_mlp_block")
-    return out
+    return (_nat or native()).mlp_block(x, w1, b1, m1, s1, gelu_c, ws.ptr, ws.nbytes, w2, b2, m2, s2, out_zp, residual, residual_rq,
+                                        w_bits, out)
 
 
 class EncoderBlock:
@@ -589,12 +569,7 @@ class EncoderBlock:
         self.ws = Workspace(int(lib().iptq_encoder_block_workspace_bytes(C.byref(p))), device)
 
     def __call__(self, x, out=None):
-        T, D = x.shape
-        if out is None:
-            out = torch.empty((T, D), dtype=torch.int8, device=x.device)
-        _chk(lib().iptq_encoder_block(_dp(x), _dp(out), C.byref(self.params), self.ws.ptr, self.ws.nbytes,
-                                      _stream()), "iptq_encoder_block")
-        return out
+        return (_nat or native()).encoder_block(x, out, self.params, self.ws.ptr, self.ws.nbytes)
 
     def profiled(self, x, out, events):
         """Same launches as ``__call__`` with ``events[0]`` recorded before the first kernel and ``events[i]``

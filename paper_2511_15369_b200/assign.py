@@ -2,10 +2,10 @@
 candidate approximation function on calibration activations, scored with the Unified Metric of Eqs. (16)-(20), and
 given the candidate with the largest term.
 
-All arithmetic runs in the library: the integer candidates are the deployed kernels (``iptq_softmax`` /
-``iptq_gelu`` / ``iptq_layernorm``), the float layer and the error sums are the ``iptq_metric_*`` reductions, the
-scoring is ``iptq_metric_term`` / ``iptq_metric_select``.  This module only sequences the calls and keeps the
-results; it synchronises with the device once, in ``finish()``.
+All arithmetic runs in the library: one ``iptq_analyze_*`` launch per layer evaluates the float layer and every integer
+candidate (on the device functions of the deployed kernels) and reduces their error sums, the scoring is
+``iptq_metric_term`` / ``iptq_metric_select``.  This module only sequences the calls and keeps the results; it
+synchronises with the device once, in ``finish()``.
 """
 from __future__ import annotations
 
@@ -21,7 +21,7 @@ GELU_CANDIDATES = (api.GELU_POLY4, api.GELU_POLY2, api.GELU_SHIFT)
 LN_CANDIDATES = (api.LN_SHIFT, api.LN_NEWTON, api.LN_PTF)
 
 
-@dataclass
+@dataclass(slots=True)
 class Candidate:
     variant: int
     op_count: float
@@ -33,7 +33,7 @@ class Candidate:
     term: float = float("nan")
 
 
-@dataclass
+@dataclass(slots=True)
 class Layer:
     name: str
     kind: int
@@ -41,103 +41,71 @@ class Layer:
     choice: int = -1               # variant id of the selected candidate
 
 
-class _Slot:
-    """MetricScratch look-alike that points one evaluation at its own row of the sums buffer."""
-
-    def __init__(self, work, sums_row):
-        self.work = work
-        self.sums = sums_row
-
-
 class Analyzer:
     def __init__(self, device="cuda", max_evaluations=256, c_unit=1.0e6):
         self.device = device
         self.c_unit = float(c_unit)
-        self.work = torch.empty(api.METRIC_WORK_BYTES // 8, dtype=torch.float64, device=device)
-        self.sums = torch.zeros((max_evaluations, 2), dtype=torch.float64, device=device)
+        self.max_evaluations = max_evaluations
+        # the scratch of the launches (its counter starts at zero) and the sums, with room for one more layer's candidates
+        # behind the last evaluation that counts
+        self._buf = torch.zeros(api.ANALYZE_WORK_BYTES // 8 + 2 * (max_evaluations + api.ANALYZE_MAX_CANDIDATES), dtype=torch.float64,
+                                device=device)
+        self.sums = self._buf[api.ANALYZE_WORK_BYTES // 8:].view(-1, 2)
+        self._work_ptr, self._sums_ptr = self._buf.data_ptr(), self.sums.data_ptr()
+        self._native = api.native()
         self.layers: list[Layer] = []
         self.n_eval = 0
-        self._keep = []            # tables referenced by raw pointers until finish()
 
-    def _slot(self):
-        if self.n_eval >= self.sums.shape[0]:
-            raise RuntimeError("more evaluations than max_evaluations")
-        s = _Slot(self.work, self.sums[self.n_eval])
-        self.n_eval += 1
-        return s
+    def _add(self, layer, variants, launch):
+        """Runs the candidates of one layer, as many per launch as a launch takes, and records them."""
+        for i in range(0, len(variants), api.ANALYZE_MAX_CANDIDATES):
+            if self.n_eval >= self.max_evaluations:
+                raise RuntimeError("more evaluations than max_evaluations")
+            done = launch(variants[i:i + api.ANALYZE_MAX_CANDIDATES], self._sums_ptr + 16 * self.n_eval, self._work_ptr)
+            for v, ops in done:
+                layer.candidates.append(Candidate(v, ops, self.n_eval))
+                self.n_eval += 1
+            if self.n_eval > self.max_evaluations:
+                raise RuntimeError("more evaluations than max_evaluations")
+        self.layers.append(layer)
+        return layer
 
     def softmax_layer(self, name, scores, in_scale, variants=SOFTMAX_CANDIDATES, out_bits=8):
-        """scores: device int32 [rows, n] at scale in_scale."""
-        rows, n = scores.shape
-        layer = Layer(name, api.LAYER_SOFTMAX)
-        probs = torch.empty((rows, n), dtype=torch.uint8, device=scores.device)
-        for v in variants:
-            bits = 4 if v == api.SM_LOG2 else out_bits         # the logarithm candidate writes 4-bit codes
-            try:
-                c = api.softmax_prepare(in_scale, n, bits, v)
-            except api.IptqError:
-                continue                   # this candidate has no integer constants at this scale
-            self._keep.append(api.softmax_table(c, scores.device))
-            api.softmax(scores, c, out=probs)
-            slot = self._slot()
-            api.metric_softmax(scores, probs, in_scale, api.PROBS_LOG2 if v == api.SM_LOG2 else bits, scratch=slot)
-            layer.candidates.append(Candidate(v, api.op_count(api.LAYER_SOFTMAX, v, rows, n), self.n_eval - 1))
-        self.layers.append(layer)
-        return layer
+        """scores: device int32 [rows, n] at scale in_scale.  A candidate that has no integer constants at this scale is left
+        out."""
+        n = self._native
+        return self._add(Layer(name, api.LAYER_SOFTMAX), variants,
+                         lambda v, sums, work: n.analyze_softmax(scores, in_scale, v, out_bits, sums, work))
 
     def gelu_layer(self, name, x, in_scale, in_bits, out_scale, out_zp, variants=GELU_CANDIDATES, out_bits=8):
-        """x: device int32 (any shape) at scale in_scale, in_bits wide."""
-        layer = Layer(name, api.LAYER_GELU)
-        y = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-        for v in variants:
-            try:
-                c = api.gelu_prepare(in_scale, in_bits, out_scale, out_zp, out_bits, v)
-            except api.IptqError:
-                continue                   # this candidate has no integer constants at this scale / width
-            api.gelu(x, c, out=y)
-            slot = self._slot()
-            api.metric_gelu(x, y, in_scale, out_scale, out_zp, scratch=slot)
-            layer.candidates.append(Candidate(v, api.op_count(api.LAYER_GELU, v, x.numel(), 1), self.n_eval - 1))
-        self.layers.append(layer)
-        return layer
+        """x: device int32 (any shape) at scale in_scale, in_bits wide.  A candidate that has no integer constants at this scale
+        and width is left out."""
+        n = self._native
+        return self._add(Layer(name, api.LAYER_GELU), variants,
+                         lambda v, sums, work: n.analyze_gelu(x, in_scale, in_bits, out_scale, out_zp, out_bits, v, sums, work))
 
     def layernorm_layer(self, name, x, gamma, beta, out_scale, out_zp, variants=LN_CANDIDATES, ptf_shift=None,
                         out_bits=8):
         """x: device int8 [rows, dim]; gamma, beta: host float32 [dim]; ptf_shift: device uint8 [dim], used by the
-        LN_PTF candidate only (the other candidates read x as it is)."""
-        rows, dim = x.shape
-        layer = Layer(name, api.LAYER_LAYERNORM)
-        g = torch.from_numpy(np.ascontiguousarray(gamma, dtype=np.float32)).to(x.device)
-        b = torch.from_numpy(np.ascontiguousarray(beta, dtype=np.float32)).to(x.device)
-        y = torch.empty((rows, dim), dtype=torch.int8, device=x.device)
-        for v in variants:
-            if v == api.LN_PTF and ptf_shift is None:
-                continue
-            gq, bq, c = api.layernorm_prepare(gamma, beta, out_scale, out_zp, out_bits, v)
-            gqd, bqd = torch.from_numpy(gq).to(x.device), torch.from_numpy(bq).to(x.device)
-            ptf = ptf_shift if v == api.LN_PTF else None
-            api.layernorm(x, gqd, bqd, c, ptf, out=y)
-            slot = self._slot()
-            api.metric_layernorm(x, y, g, b, out_scale, out_zp, ptf, scratch=slot)
-            layer.candidates.append(Candidate(v, api.op_count(api.LAYER_LAYERNORM, v, rows, dim), self.n_eval - 1))
-        self.layers.append(layer)
-        return layer
+        LN_PTF candidate only (the other candidates read x as it is; without it the LN_PTF candidate is left out)."""
+        n = self._native
+        g, b = np.ascontiguousarray(gamma, dtype=np.float32), np.ascontiguousarray(beta, dtype=np.float32)
+        return self._add(Layer(name, api.LAYER_LAYERNORM), variants,
+                         lambda v, sums, work: n.analyze_layernorm(x, g, b, out_scale, out_zp, out_bits, v, ptf_shift, sums, work))
 
     def finish(self):
         """Reads the sums back (the only synchronisation), scores every candidate and selects per layer.
         Returns (layers, Omega) with Omega the sum of the selected terms, Eq. (16)."""
-        host = self.sums[:max(self.n_eval, 1)].cpu().numpy()
+        host = self.sums[:max(self.n_eval, 1)].cpu()
+        ptr = host.data_ptr()
         omega = 0.0
         for layer in self.layers:
-            for cand in layer.candidates:
-                cand.sum_x2, cand.sum_err2 = float(host[cand.slot, 0]), float(host[cand.slot, 1])
-                cand.sqnr_db = api.sqnr_db(cand.sum_x2, cand.sum_err2)
+            cands = layer.candidates
+            best, scores = self._native.metric_scores(ptr, cands[0].slot if cands else 0, [c.op_count for c in cands], self.c_unit)
+            for cand, (cand.sum_x2, cand.sum_err2, cand.sqnr_db, cand.term) in zip(cands, scores):
                 cand.perturbation = cand.sum_err2
-                cand.term = api.metric_term(cand.sqnr_db, cand.perturbation, cand.op_count, self.c_unit)
-            best = api.metric_select([c.term for c in layer.candidates])
-            layer.choice = layer.candidates[best].variant
-            omega += layer.candidates[best].term
-        self._keep.clear()
+            layer.choice = cands[best].variant
+            omega += cands[best].term
         return self.layers, omega
 
 

@@ -1,4 +1,5 @@
-"""Builds the CUDA library in-tree: every csrc/*.cu -> object -> libiptq.so (sm_100a only)."""
+"""Builds the CUDA library in-tree: every csrc/*.cu -> object -> libiptq.so (sm_100a only), and the native half of the
+Python binding, csrc/binding.cpp -> _native.so (against the installed torch)."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -12,6 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libiptq.so")
+NATIVE = os.path.join(HERE, "_native.so")
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,6 +25,21 @@ def _stale(target: str, deps: list[str]) -> bool:
         return True
     t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _native_cmd(src: str, out: str) -> list[str]:
+    import sysconfig
+
+    import torch
+    t = os.path.dirname(torch.__file__)
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), src, "-o", out]
+    for d in (os.path.join(ROOT, "include"), os.path.join(t, "include"), os.path.join(t, "include", "torch", "csrc", "api", "include"),
+              "/usr/local/cuda/include", sysconfig.get_paths()["include"]):
+        cmd += ["-isystem", d]
+    lib = os.path.join(t, "lib")
+    cudart = sorted(glob.glob(os.path.join(os.path.dirname(t), "nvidia", "*", "lib", "libcudart.so.1*")))
+    return cmd + ["-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"] + cudart[:1]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -37,12 +54,19 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if force or _stale(obj, [src] + headers):
             cmd = [NVCC] + FLAGS + (["-Xptxas", "-v"] if verbose else []) + ["-c", src, "-o", obj]
             jobs.append(cmd)
+    binding = os.path.join(CSRC, "binding.cpp")
+    native_tmp = None
+    if force or _stale(NATIVE, [binding, os.path.join(ROOT, "include", "iptq.h")]):
+        native_tmp = NATIVE + ".tmp.%d" % os.getpid()
+        jobs.append(_native_cmd(binding, native_tmp))
     with concurrent.futures.ThreadPoolExecutor(max_workers=8) as ex:
         for cmd, res in zip(jobs, ex.map(lambda c: subprocess.run(c, capture_output=True, text=True), jobs)):
             if verbose or res.returncode != 0:
                 sys.stderr.write(" ".join(cmd) + "\n" + res.stdout + res.stderr)
             if res.returncode != 0:
-                raise RuntimeError("nvcc failed on " + cmd[-3])
+                raise RuntimeError("compilation failed: " + " ".join(cmd))
+    if native_tmp:
+        os.replace(native_tmp, NATIVE)
     if jobs or force or _stale(LIB, objs):
         tmp = LIB + ".tmp.%d" % os.getpid()
         subprocess.check_call([NVCC, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])

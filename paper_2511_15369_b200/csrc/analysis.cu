@@ -1,0 +1,421 @@
+// Unified-Metric analysis of one layer (Sec. 3.5): every candidate function of the layer and the float layer in one pass
+// over its calibration activations, reduced to (sum X^2, sum (X - Q)^2) per candidate.
+//
+// One launch per layer.  Launched as the candidates' own kernels followed by iptq_metric_*() -- four launches per
+// candidate, the integer output written and read again, the float layer (fp64 exp or erf) evaluated once per
+// candidate -- the 159 evaluations of a DeiT-Small encoder at batch 8 kept the device busy for 3.5 ms and the host for
+// 9.7 ms.  Here the activations are read once, the float layer is evaluated once and the candidates run in registers on
+// the device functions of the deployed kernels, so their integers are the same.
+#include <climits>
+#include <cmath>
+
+#include "iptq_common.cuh"
+
+namespace iptq {
+
+constexpr unsigned kAllLanes = 0xffffffffu;
+constexpr int kAnThreads = 256;
+constexpr int kAnMaxCand = IPTQ_ANALYZE_MAX_CANDIDATES;
+constexpr int kAnMaxBlocks = (IPTQ_ANALYZE_WORK_BYTES - 256) / (16 * kAnMaxCand);
+
+__device__ __forceinline__ double an_warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kAllLanes, v, o);
+    return v;
+}
+
+// An int32 as a double without the conversion unit: 2^52 + 2^31 + v in the bits, both offsets subtracted.
+__device__ __forceinline__ double an_to_double(int v)
+{
+    return __hiloint2double(0x43300000, v ^ (int)0x80000000) - 4503601774854144.0;
+}
+
+// Adds the CTAs' pairs (x2[i], e2[i]), i < n, in an order that depends on the launch alone: lanes by butterfly, warps and
+// CTAs in index order.  The CTA that finishes last does the final sum and leaves the counter at zero.
+__device__ __forceinline__ void an_finish(const double (&x2)[kAnMaxCand], const double (&e2)[kAnMaxCand], int n, double* sums,
+                                          unsigned* counter, double* partials)
+{
+    __shared__ double sh[2 * kAnMaxCand][kAnThreads / 32];
+    __shared__ bool last;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < kAnMaxCand; ++i) {
+        if (i < n) {
+            const double a = an_warp_sum(x2[i]), b = an_warp_sum(e2[i]);
+            if (lane == 0) { sh[2 * i][w] = a; sh[2 * i + 1][w] = b; }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * n) {
+        double t = 0.0;
+        for (int i = 0; i < kAnThreads / 32; ++i) t += sh[threadIdx.x][i];
+        partials[(size_t)blockIdx.x * 2 * kAnMaxCand + threadIdx.x] = t;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int i = w; i < 2 * n; i += kAnThreads / 32) {
+        double t = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(partials + (size_t)b * 2 * kAnMaxCand + i);
+        t = an_warp_sum(t);
+        if (lane == 0) sums[i] = t;
+    }
+    if (threadIdx.x == 0) *counter = 0;
+}
+
+// ------------------------------------------------------------------------------------------------ Softmax
+struct AnSoftmaxCand {
+    ExpDev ex;
+    int variant, M, f_shl, p_shr;
+    double step;                       // value of one unit of the output byte (linear candidates)
+};
+struct AnSoftmax {
+    AnSoftmaxCand c[kAnMaxCand];
+};
+
+template <int VARIANT, int NITER>
+__device__ __forceinline__ double an_softmax_err(const AnSoftmaxCand& c, const int (&v)[NITER], const double (&X)[NITER], int mx)
+{
+    unsigned e[NITER];
+    unsigned sum = 0;
+#pragma unroll
+    for (int k = 0; k < NITER; ++k) {
+        e[k] = exp_core_nd<VARIANT>(exp_distance(mx, v[k]), c.ex);       // 0 for lanes past the row end
+        sum += e[k];
+    }
+    sum = __reduce_add_sync(kAllLanes, sum);
+    const unsigned f = VARIANT == IPTQ_SM_LOG2 ? 0u : intdiv_factor(sum, c.M) << c.f_shl;
+    double err = 0.0;
+#pragma unroll
+    for (int k = 0; k < NITER; ++k) {
+        double q;
+        if (VARIANT == IPTQ_SM_LOG2) {
+            const unsigned code = log2_code(sum, e[k]);
+            q = code == IPTQ_LOG2_ZERO ? 0.0 : __hiloint2double((int)(1023u - code) << 20, 0);
+        } else {
+            q = an_to_double((int)(__umulhi(f, e[k]) >> c.p_shr)) * c.step;
+        }
+        const double d = X[k] - q;
+        err = fma(d, d, err);
+    }
+    return err;
+}
+
+// A warp per row, the row and its float Softmax in registers.
+template <int NITER>
+__global__ void __launch_bounds__(kAnThreads)
+analyze_softmax_kernel(const int32_t* __restrict__ scores, int64_t rows, int n, double in_scale, const __grid_constant__ AnSoftmax a,
+                       int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter, double* __restrict__ partials)
+{
+    grid_dep_launch();
+    grid_dep_wait();
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (int64_t)blockIdx.x * (kAnThreads >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarps = (int64_t)gridDim.x * (kAnThreads >> 5);
+    const int iters = (n + 31) >> 5;                                     // <= NITER
+    double x2 = 0.0, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t row = warp; row < rows; row += nwarps) {
+        const int32_t* sr = scores + row * n + lane;
+        int v[NITER];
+        int mx = INT_MIN;
+#pragma unroll
+        for (int k = 0; k < NITER; ++k) {
+            v[k] = lane + 32 * k < n ? __ldg(sr + 32 * k) : kNoScore;
+            mx = max(mx, v[k]);
+        }
+        mx = __reduce_max_sync(kAllLanes, mx);
+        const double zmax = (double)mx * in_scale;
+        double X[NITER];
+        double den = 0.0;
+#pragma unroll
+        for (int k = 0; k < NITER; ++k) {
+            X[k] = 0.0;
+            if (k < iters) {                                             // uniform
+                if (lane + 32 * k < n) X[k] = exp(fma(an_to_double(v[k]), in_scale, -zmax));
+                den += X[k];
+            }
+        }
+        const double inv = 1.0 / an_warp_sum(den);
+#pragma unroll
+        for (int k = 0; k < NITER; ++k) {
+            X[k] *= inv;
+            x2 = fma(X[k], X[k], x2);
+        }
+        // every element past the row end has X = 0 and an integer probability of 0, except a logarithm code of such a lane,
+        // which is IPTQ_LOG2_ZERO = probability 0 as well
+        for (int i = 0; i < n_cand; ++i) {
+            const AnSoftmaxCand& c = a.c[i];
+            double err;
+            switch (c.variant) {
+                case IPTQ_SM_BITEXP: err = an_softmax_err<IPTQ_SM_BITEXP, NITER>(c, v, X, mx); break;
+                case IPTQ_SM_SHIFTMAX: err = an_softmax_err<IPTQ_SM_SHIFTMAX, NITER>(c, v, X, mx); break;
+                case IPTQ_SM_POLY: err = an_softmax_err<IPTQ_SM_POLY, NITER>(c, v, X, mx); break;
+                default: err = an_softmax_err<IPTQ_SM_LOG2, NITER>(c, v, X, mx); break;
+            }
+#pragma unroll
+            for (int j = 0; j < kAnMaxCand; ++j) e2[j] += j == i ? err : 0.0;
+        }
+    }
+    const double xs[kAnMaxCand] = {x2, x2, x2, x2};
+    an_finish(xs, e2, n_cand, sums, counter, partials);
+}
+
+// ------------------------------------------------------------------------------------------------ GELU
+struct AnGelu {
+    GeluDev c[kAnMaxCand];
+};
+
+__device__ __forceinline__ int an_gelu(int x, const GeluDev& c)
+{
+    switch (c.variant) {
+        case IPTQ_GELU_POLY4: return requant_full(gelu_core<IPTQ_GELU_POLY4>(x, c), c.out);
+        case IPTQ_GELU_POLY2: return requant_full(gelu_core<IPTQ_GELU_POLY2>(x, c), c.out);
+        default: return requant_full(gelu_core<IPTQ_GELU_SHIFT>(x, c), c.out);
+    }
+}
+
+__global__ void __launch_bounds__(kAnThreads)
+analyze_gelu_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, double out_scale, int out_zp,
+                    const __grid_constant__ AnGelu a, int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter,
+                    double* __restrict__ partials)
+{
+    grid_dep_launch();
+    grid_dep_wait();
+    double x2 = 0.0, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
+    auto element = [&](int xi) {
+        const double v = an_to_double(xi) * in_scale;
+        const double X = 0.5 * v * (1.0 + erf(v * 0.70710678118654752440));
+        x2 = fma(X, X, x2);
+#pragma unroll
+        for (int i = 0; i < kAnMaxCand; ++i) {
+            if (i < n_cand) {
+                const double d = X - an_to_double(an_gelu(xi, a.c[i]) - out_zp) * out_scale;
+                e2[i] = fma(d, d, e2[i]);
+            }
+        }
+    };
+    const int64_t nvec = n >> 2, stride = (int64_t)gridDim.x * kAnThreads, first = (int64_t)blockIdx.x * kAnThreads + threadIdx.x;
+    const int4* xv = reinterpret_cast<const int4*>(x);
+    for (int64_t i = first; i < nvec; i += stride) {
+        const int4 q = __ldg(xv + i);
+        element(q.x); element(q.y); element(q.z); element(q.w);
+    }
+    if ((nvec << 2) + first < n) element(__ldg(x + (nvec << 2) + first));
+    const double xs[kAnMaxCand] = {x2, x2, x2, x2};
+    an_finish(xs, e2, n_cand, sums, counter, partials);
+}
+
+// ------------------------------------------------------------------------------------------------ LayerNorm
+struct AnLayerNorm {
+    int variant[kAnMaxCand];
+    RequantDev out[kAnMaxCand];
+};
+
+// A warp per row, under two readings of its input: index 0 plain, 1 with the power-of-two factors.  The row is read twice (the
+// second time from L1); the float parameters wait in shared memory as doubles.
+__global__ void __launch_bounds__(kAnThreads)
+analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, const float* __restrict__ gamma,
+                         const float* __restrict__ beta, const int32_t* __restrict__ gamma_q, const int32_t* __restrict__ beta_q,
+                         const uint8_t* __restrict__ ptf, double out_scale, int out_zp, const __grid_constant__ AnLayerNorm a,
+                         int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter, double* __restrict__ partials)
+{
+    extern __shared__ __align__(16) double gb[];                         // gamma[D], beta[D]
+    grid_dep_launch();
+    grid_dep_wait();
+    for (int i = threadIdx.x; i < D; i += kAnThreads) { gb[i] = (double)__ldg(gamma + i); gb[D + i] = (double)__ldg(beta + i); }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, words = D >> 2;
+    const int64_t warp = (int64_t)blockIdx.x * (kAnThreads >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarps = (int64_t)gridDim.x * (kAnThreads >> 5);
+    bool any_plain = false, any_ptf = false;
+    for (int i = 0; i < n_cand; ++i) { any_ptf |= a.variant[i] == IPTQ_LN_PTF; any_plain |= a.variant[i] != IPTQ_LN_PTF; }
+    double x2[2] = {0.0, 0.0}, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t row = warp; row < rows; row += nwarps) {
+        const int* xr = reinterpret_cast<const int*>(x + row * D);
+        int s1[2] = {0, 0};
+        unsigned s2[2] = {0, 0};
+        for (int wi = lane; wi < words; wi += 32) {
+            const int w = __ldg(xr + wi);
+            if (any_plain) {
+                s1[0] = __dp4a(w, 0x01010101, s1[0]);
+                s2[0] = (unsigned)__dp4a(w, w, (int)s2[0]);
+            }
+            if (any_ptf) {
+                const unsigned sh = __ldg(reinterpret_cast<const unsigned*>(ptf) + wi);
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int xv = ((int)(int8_t)(w >> (8 * t))) << ((sh >> (8 * t)) & 3);
+                    s1[1] += xv;
+                    s2[1] += (unsigned)(xv * xv);
+                }
+            }
+        }
+        double mu[2], inv_sd[2];
+        long long F[kAnMaxCand];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            s1[p] = __reduce_add_sync(kAllLanes, s1[p]);
+            s2[p] = __reduce_add_sync(kAllLanes, s2[p]);
+            const long long V = (long long)D * (long long)s2[p] - (long long)s1[p] * (long long)s1[p];    // D^2 var
+            mu[p] = (double)s1[p] / (double)D;
+            inv_sd[p] = V > 0 ? (double)D / sqrt((double)V) : 0.0;       // a constant row gives beta
+#pragma unroll
+            for (int i = 0; i < kAnMaxCand; ++i) {
+                if (i < n_cand && (a.variant[i] == IPTQ_LN_PTF) == (p == 1)) {
+                    const unsigned long long rt = ln_isqrt((unsigned long long)V, a.variant[i]);
+                    F[i] = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;
+                }
+            }
+        }
+        for (int wi = lane; wi < words; wi += 32) {
+            const unsigned w = (unsigned)__ldg(xr + wi);
+            const unsigned sh = any_ptf ? __ldg(reinterpret_cast<const unsigned*>(ptf) + wi) : 0u;
+            const int4 g4 = __ldg(reinterpret_cast<const int4*>(gamma_q) + wi), b4 = __ldg(reinterpret_cast<const int4*>(beta_q) + wi);
+            const int gq[4] = {g4.x, g4.y, g4.z, g4.w}, bq[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int xv[2] = {(int)(int8_t)(w >> (8 * t)), ((int)(int8_t)(w >> (8 * t))) << ((sh >> (8 * t)) & 3)};
+                const double ga = gb[4 * wi + t], be = gb[D + 4 * wi + t];
+                double X[2] = {0.0, 0.0};
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    if (p == 0 ? any_plain : any_ptf) {
+                        X[p] = fma((an_to_double(xv[p]) - mu[p]) * inv_sd[p], ga, be);
+                        x2[p] = fma(X[p], X[p], x2[p]);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < kAnMaxCand; ++i) {
+                    if (i < n_cand) {
+                        const int p = a.variant[i] == IPTQ_LN_PTF ? 1 : 0;
+                        const int u = D * (p ? xv[1] : xv[0]) - (p ? s1[1] : s1[0]);
+                        const int nq = (int)(((long long)u * F[i]) >> 30);
+                        const int o = requant_full(nq * gq[t] + bq[t], a.out[i]);
+                        const double d = (p ? X[1] : X[0]) - an_to_double(o - out_zp) * out_scale;
+                        e2[i] = fma(d, d, e2[i]);
+                    }
+                }
+            }
+        }
+    }
+    double xs[kAnMaxCand];
+#pragma unroll
+    for (int i = 0; i < kAnMaxCand; ++i) xs[i] = i < n_cand && a.variant[i] == IPTQ_LN_PTF ? x2[1] : x2[0];
+    an_finish(xs, e2, n_cand, sums, counter, partials);
+}
+
+static int an_grid(int64_t blocks)
+{
+    return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, std::min<int64_t>((int64_t)sm_count() * 4, kAnMaxBlocks)));
+}
+
+static int an_args_ok(const void* consts, int n_cand, const void* sums, const void* work)
+{
+    if (!consts || !sums || !work) return IPTQ_ERR_NULL;
+    if (n_cand < 1 || n_cand > kAnMaxCand) return IPTQ_ERR_SHAPE;
+    if (!aligned16(sums) || !aligned16(work)) return IPTQ_ERR_ALIGN;
+    return IPTQ_OK;
+}
+
+}  // namespace iptq
+
+using namespace iptq;
+
+extern "C" {
+
+int iptq_analyze_softmax(const int32_t* scores, int64_t rows, int row_len, double in_scale, const iptq_softmax_consts* consts,
+                         int n_candidates, double* sums, void* work, iptq_stream_t stream)
+{
+    int rc = an_args_ok(consts, n_candidates, sums, work);
+    if (rc != IPTQ_OK) return rc;
+    if (rows < 0 || row_len < 1 || row_len > 1024) return IPTQ_ERR_SHAPE;
+    if (!(in_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
+    if (rows > 0 && !scores) return IPTQ_ERR_NULL;
+    if (!aligned16(scores)) return IPTQ_ERR_ALIGN;
+    AnSoftmax a{};
+    for (int i = 0; i < n_candidates; ++i) {
+        const iptq_softmax_consts& c = consts[i];
+        if (c.row_len != row_len) return IPTQ_ERR_SHAPE;
+        if (c.out_bits < 4 || c.out_bits > 8) return IPTQ_ERR_BITS;
+        if (c.x0 < 8 || c.M < 31 || c.M > 40) return IPTQ_ERR_SCALE_RANGE;
+        if (c.variant < 0 || c.variant > 3) return IPTQ_ERR_VARIANT;
+        a.c[i].ex = to_dev_exp(c);
+        a.c[i].variant = c.variant; a.c[i].M = c.M; a.c[i].f_shl = c.f_shl; a.c[i].p_shr = c.p_shr;
+        a.c[i].step = 1.0 / (double)(1 << (c.out_bits - 1));
+    }
+    unsigned* counter = static_cast<unsigned*>(work);
+    double* partials = reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256);
+    const int grid = an_grid((rows + 7) / 8), it = (row_len + 31) / 32;
+#define IPTQ_AN_SM(NI)                                                                                                    \
+    launch_kernel(analyze_softmax_kernel<NI>, grid, kAnThreads, 0, stream, scores, rows, row_len, in_scale, a, n_candidates, \
+                  sums, counter, partials)
+    if (it <= 2) IPTQ_AN_SM(2);
+    else if (it <= 4) IPTQ_AN_SM(4);
+    else if (it <= 5) IPTQ_AN_SM(5);
+    else if (it <= 7) IPTQ_AN_SM(7);
+    else if (it <= 8) IPTQ_AN_SM(8);
+    else if (it <= 16) IPTQ_AN_SM(16);
+    else IPTQ_AN_SM(32);
+#undef IPTQ_AN_SM
+    note_launch();
+    return last_launch_status();
+}
+
+int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_scale, int out_zp,
+                      const iptq_gelu_consts* consts, int n_candidates, double* sums, void* work, iptq_stream_t stream)
+{
+    int rc = an_args_ok(consts, n_candidates, sums, work);
+    if (rc != IPTQ_OK) return rc;
+    if (n < 0) return IPTQ_ERR_SHAPE;
+    if (!(in_scale > 0.0) || !(out_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
+    if (n > 0 && !x) return IPTQ_ERR_NULL;
+    if (!aligned16(x)) return IPTQ_ERR_ALIGN;
+    AnGelu a{};
+    for (int i = 0; i < n_candidates; ++i) {
+        if (consts[i].in_bits < 8 || consts[i].in_bits > 16) return IPTQ_ERR_BITS;
+        if (consts[i].variant < 0 || consts[i].variant > 2) return IPTQ_ERR_VARIANT;
+        if ((rc = check_requant(&consts[i].out)) != IPTQ_OK) return rc;
+        a.c[i] = to_dev(consts[i]);
+    }
+    launch_kernel(analyze_gelu_kernel, an_grid((n / 4 + kAnThreads - 1) / kAnThreads), kAnThreads, 0, stream, x, n, in_scale,
+                  out_scale, out_zp, a, n_candidates, sums, static_cast<unsigned*>(work),
+                  reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256));
+    note_launch();
+    return last_launch_status();
+}
+
+int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* gamma, const float* beta,
+                           const int32_t* gamma_q, const int32_t* beta_q, const uint8_t* ptf_shift, double out_scale,
+                           int out_zp, const iptq_ln_consts* consts, int n_candidates, double* sums, void* work,
+                           iptq_stream_t stream)
+{
+    int rc = an_args_ok(consts, n_candidates, sums, work);
+    if (rc != IPTQ_OK) return rc;
+    if (rows < 0 || dim < 4 || dim > 3072 || (dim & 3)) return IPTQ_ERR_SHAPE;
+    if (!(out_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
+    if (!gamma || !beta || !gamma_q || !beta_q || (rows > 0 && !x)) return IPTQ_ERR_NULL;
+    if (!aligned16(x) || !aligned16(gamma_q) || !aligned16(beta_q) || (reinterpret_cast<uintptr_t>(ptf_shift) & 3u)) return IPTQ_ERR_ALIGN;
+    AnLayerNorm a{};
+    for (int i = 0; i < n_candidates; ++i) {
+        if (consts[i].dim != dim) return IPTQ_ERR_SHAPE;
+        if (consts[i].variant < 0 || consts[i].variant > 2) return IPTQ_ERR_VARIANT;
+        if (consts[i].variant == IPTQ_LN_PTF && !ptf_shift) return IPTQ_ERR_NULL;
+        if ((rc = check_requant(&consts[i].out)) != IPTQ_OK) return rc;
+        a.variant[i] = consts[i].variant;
+        a.out[i] = to_dev(consts[i].out);
+    }
+    // 16 bytes per channel beside the static shared memory: wide rows pass the default limit of 48 KB
+    if (dim > 2048 && cudaFuncSetAttribute(analyze_layernorm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 3072) != cudaSuccess)
+        return IPTQ_ERR_CUDA;
+    launch_kernel(analyze_layernorm_kernel, an_grid((rows + 7) / 8), kAnThreads, (size_t)16 * dim, stream, x, rows, dim, gamma,
+                  beta, gamma_q, beta_q, ptf_shift, out_scale, out_zp, a, n_candidates, sums, static_cast<unsigned*>(work),
+                  reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256));
+    note_launch();
+    return last_launch_status();
+}
+
+}  // extern "C"

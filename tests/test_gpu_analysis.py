@@ -1,0 +1,97 @@
+"""The one-launch-per-layer analysis (iptq_analyze_*) against the numpy oracle of the Unified Metric at the sizes where its
+kernels can go wrong: rows shorter than a warp step, at and past a step's end, element counts that are no multiple of a
+vector, the widest rows.  Tolerance as for iptq_metric_*: fp64 sums in another order and another exp / erf move them by
+about 1e-13; 1e-9 relative leaves four orders of margin."""
+import numpy as np
+import pytest
+
+from paper_2511_15369_b200 import synth
+
+pytestmark = pytest.mark.gpu
+REL = 1e-9
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from oracle import metric
+    from paper_2511_15369_b200 import api, assign
+    api.lib()
+    return api, assign, metric
+
+
+def _cu(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _same(cand, want):
+    assert abs(cand.sum_x2 - want[0]) <= REL * abs(want[0]), (cand, want)
+    assert abs(cand.sum_err2 - want[1]) <= REL * abs(want[1]), (cand, want)
+
+
+@pytest.mark.parametrize("rows,n", [(1, 1), (3, 32), (9, 33), (70, 64), (11, 65), (300, 129), (591, 197), (40, 256), (17, 257), (5, 512), (9, 1000)])
+def test_softmax_candidates(env, orc, rows, n):
+    api, assign, metric = env
+    S = synth.SOFTMAX_SCALE_ACC
+    s = synth.quantize_scores(synth.softmax_logits(rows, n, seed=rows + n), S)
+    an = assign.Analyzer()
+    layer = an.softmax_layer("x", _cu(s), S)
+    an.finish()
+    X = metric.softmax_float(s, S)
+    assert [c.variant for c in layer.candidates] == [0, 1, 2, 3]
+    for c in layer.candidates:
+        p = orc.softmax(s, orc.softmax_prepare(S, n, 4 if c.variant == orc.SM_LOG2 else 8, c.variant))
+        _same(c, metric.error_sums(X, metric.log2_deq(p) if c.variant == orc.SM_LOG2 else metric.softmax_deq(p, 8)))
+        assert c.op_count == api.op_count(api.LAYER_SOFTMAX, c.variant, rows, n)
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 1023, 4097, 1 << 18])
+def test_gelu_candidates(env, orc, n):
+    api, assign, metric = env
+    S = 2.5e-4
+    xq = np.clip(np.round(synth.gelu_values(n, seed=n) / S), -32768, 32767).astype(np.int32)
+    So, zp = 8.2 / 255, -123
+    an = assign.Analyzer()
+    layer = an.gelu_layer("x", _cu(xq), S, 16, So, zp)
+    an.finish()
+    assert [c.variant for c in layer.candidates] == [0, 1, 2]
+    for c in layer.candidates:
+        y = orc.gelu(xq, orc.gelu_prepare(S, 16, So, zp, 8, c.variant))
+        _same(c, metric.error_sums(metric.gelu_float(xq, S), metric.affine_deq(y, So, zp)))
+
+
+@pytest.mark.parametrize("rows,dim", [(1, 4), (9, 100), (33, 128), (197, 192), (50, 768), (7, 3072)])
+def test_layernorm_candidates(env, orc, rows, dim):
+    api, assign, metric = env
+    xf, gamma, beta, _ = synth.ln_values(rows, dim, seed=dim)
+    x, _ = synth.quantize_sym(xf, 8, np.int8)
+    if rows > 2:
+        x[2] = 5                                               # a constant row
+    ptf = (np.arange(dim) % 4).astype(np.uint8)
+    So, zp = 8.0 / 127, 3
+    an = assign.Analyzer()
+    layer = an.layernorm_layer("x", _cu(x), gamma, beta, So, zp, ptf_shift=_cu(ptf))
+    an.finish()
+    assert [c.variant for c in layer.candidates] == [0, 1, 2]
+    for c in layer.candidates:
+        gq, bq, oc = orc.layernorm_prepare(gamma, beta, So, zp, 8, c.variant)
+        sh = ptf if c.variant == orc.LN_PTF else None
+        y = orc.layernorm(x, gq, bq, oc, sh)
+        _same(c, metric.error_sums(metric.layernorm_float(x, gamma, beta, sh), metric.affine_deq(y, So, zp)))
+
+
+def test_sums_are_the_same_bits_twice_and_the_capacity_is_kept(env):
+    api, assign, metric = env
+    S = synth.SOFTMAX_SCALE_ACC
+    s = _cu(synth.quantize_scores(synth.softmax_logits(1000, 197, seed=1), S))
+    an = assign.Analyzer(max_evaluations=8)
+    for _ in range(2):
+        an.softmax_layer("x", s, S)
+    with pytest.raises(RuntimeError):
+        an.softmax_layer("x", s, S)
+    a, b = an.layers
+    an.finish()
+    assert [(c.sum_x2, c.sum_err2) for c in a.candidates] == [(c.sum_x2, c.sum_err2) for c in b.candidates]

@@ -401,19 +401,20 @@ int iptq_metric_layernorm(const int8_t* x, const int8_t* y, int64_t rows, int di
  * activations): the activations are read once, the float layer is evaluated once, the candidates' integer outputs stay
  * in registers.  The integers are those of iptq_softmax() / iptq_gelu() / iptq_layernorm() with the same constants;
  * the summation order is fixed for a device and sizes but is not that of iptq_metric_*().
- * consts: host array of n_candidates (1 .. IPTQ_ANALYZE_MAX_CANDIDATES) constants; sums: dev double [n_candidates][2], 16-byte
+ * consts: host array of n_candidates (1 .. IPTQ_ANALYZE_MAX_CANDIDATES; GELU: 1 .. 3) constants; sums: dev double [n_candidates][2], 16-byte
  * aligned; work: dev, IPTQ_ANALYZE_WORK_BYTES, 16-byte aligned, its first 4 bytes zero before the first call that uses it
- * (every call leaves them zero).  Tables in the constants are not used.  LayerNorm: gamma_q / beta_q are those of
- * iptq_layernorm_prepare() (they do not depend on the variant); ptf_shift is used by IPTQ_LN_PTF candidates alone. */
+ * (every call leaves them zero).  Tables in the constants are not used.  LayerNorm: gamma, beta, gamma_q and beta_q are HOST
+ * arrays [dim], read during the call: the float parameters and those of iptq_layernorm_prepare() (they do not depend
+ * on the variant); ptf_shift (dev) is used by IPTQ_LN_PTF candidates alone. */
 #define IPTQ_ANALYZE_MAX_CANDIDATES 4
-#define IPTQ_ANALYZE_WORK_BYTES 65536
+#define IPTQ_ANALYZE_WORK_BYTES (131072 + 32 * 65536)
 int iptq_analyze_softmax(const int32_t* scores, int64_t rows, int row_len, double in_scale,
                          const iptq_softmax_consts* consts, int n_candidates, double* sums, void* work,
                          iptq_stream_t stream);
 int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_scale, int out_zp,
                       const iptq_gelu_consts* consts, int n_candidates, double* sums, void* work, iptq_stream_t stream);
-int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* gamma, const float* beta,
-                           const int32_t* gamma_q, const int32_t* beta_q, const uint8_t* ptf_shift, double out_scale,
+int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* gamma /*host*/, const float* beta /*host*/,
+                           const int32_t* gamma_q /*host*/, const int32_t* beta_q /*host*/, const uint8_t* ptf_shift, double out_scale,
                            int out_zp, const iptq_ln_consts* consts, int n_candidates, double* sums, void* work,
                            iptq_stream_t stream);
 

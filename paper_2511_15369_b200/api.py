@@ -349,7 +349,7 @@ def gelu_table(consts: GeluConsts, device="cuda"):
 
 LAYER_SOFTMAX, LAYER_GELU, LAYER_LAYERNORM = 0, 1, 2
 METRIC_WORK_BYTES = 32768
-ANALYZE_WORK_BYTES = 65536
+ANALYZE_WORK_BYTES = 131072 + 32 * 65536
 ANALYZE_MAX_CANDIDATES = 4
 
 

@@ -48,20 +48,21 @@ class Analyzer:
         self.max_evaluations = max_evaluations
         # the scratch of the launches (its counter starts at zero) and the sums, with room for one more layer's candidates
         # behind the last evaluation that counts
-        self._buf = torch.zeros(api.ANALYZE_WORK_BYTES // 8 + 2 * (max_evaluations + api.ANALYZE_MAX_CANDIDATES), dtype=torch.float64,
+        self._buf = torch.empty(api.ANALYZE_WORK_BYTES // 8 + 2 * (max_evaluations + api.ANALYZE_MAX_CANDIDATES), dtype=torch.float64,
                                 device=device)
+        self._buf[0] = 0
         self.sums = self._buf[api.ANALYZE_WORK_BYTES // 8:].view(-1, 2)
         self._work_ptr, self._sums_ptr = self._buf.data_ptr(), self.sums.data_ptr()
         self._native = api.native()
         self.layers: list[Layer] = []
         self.n_eval = 0
 
-    def _add(self, layer, variants, launch):
+    def _add(self, layer, variants, launch, per_launch=api.ANALYZE_MAX_CANDIDATES):
         """Runs the candidates of one layer, as many per launch as a launch takes, and records them."""
-        for i in range(0, len(variants), api.ANALYZE_MAX_CANDIDATES):
+        for i in range(0, len(variants), per_launch):
             if self.n_eval >= self.max_evaluations:
                 raise RuntimeError("more evaluations than max_evaluations")
-            done = launch(variants[i:i + api.ANALYZE_MAX_CANDIDATES], self._sums_ptr + 16 * self.n_eval, self._work_ptr)
+            done = launch(variants[i:i + per_launch], self._sums_ptr + 16 * self.n_eval, self._work_ptr)
             for v, ops in done:
                 layer.candidates.append(Candidate(v, ops, self.n_eval))
                 self.n_eval += 1
@@ -82,7 +83,7 @@ class Analyzer:
         and width is left out."""
         n = self._native
         return self._add(Layer(name, api.LAYER_GELU), variants,
-                         lambda v, sums, work: n.analyze_gelu(x, in_scale, in_bits, out_scale, out_zp, out_bits, v, sums, work))
+                         lambda v, sums, work: n.analyze_gelu(x, in_scale, in_bits, out_scale, out_zp, out_bits, v, sums, work), 3)
 
     def layernorm_layer(self, name, x, gamma, beta, out_scale, out_zp, variants=LN_CANDIDATES, ptf_shift=None,
                         out_bits=8):

@@ -8,6 +8,7 @@
 // the device functions of the deployed kernels, so their integers are the same.
 #include <climits>
 #include <cmath>
+#include <cstring>
 
 #include "iptq_common.cuh"
 
@@ -16,7 +17,9 @@ namespace iptq {
 constexpr unsigned kAllLanes = 0xffffffffu;
 constexpr int kAnThreads = 256;
 constexpr int kAnMaxCand = IPTQ_ANALYZE_MAX_CANDIDATES;
-constexpr int kAnMaxBlocks = (IPTQ_ANALYZE_WORK_BYTES - 256) / (16 * kAnMaxCand);
+// scratch: the counter (256 bytes), the CTAs' pairs, the GELU terms
+constexpr int kAnPartialBytes = 131072;
+constexpr int kAnMaxBlocks = (kAnPartialBytes - 256) / (16 * kAnMaxCand);
 
 __device__ __forceinline__ double an_warp_sum(double v)
 {
@@ -105,13 +108,39 @@ __device__ __forceinline__ double an_softmax_err(const AnSoftmaxCand& c, const i
     return err;
 }
 
+// exp(-d S) of an integer distance d >= 0 as the product of two tabulated exponentials, exp(-(d >> k) 2^k S) exp(-(d mod 2^k) S):
+// two shared-memory reads and a multiply (half a unit in the last place more than exp() itself) instead of some fifty
+// fp64 instructions.  The tables cover d S < kAnExpRange, beyond which the exponential is below 1e-30 and counts as 0.
+constexpr double kAnExpRange = 70.0;
+constexpr int kAnExpMaxEntries = 4096;
+struct AnExp {
+    int shift, n_hi;                   // n_hi = 0: no tables (scales below about 1e-5), exp() per element
+};
+static AnExp an_exp(double in_scale)
+{
+    AnExp t{0, 0};
+    const double n = kAnExpRange / in_scale + 1.0;
+    while (t.shift < 30 && (double)(1 << t.shift) * (double)(1 << t.shift) < n) ++t.shift;
+    const double hi = n / (double)(1 << t.shift) + 1.0;
+    if (hi + (double)(1 << t.shift) <= (double)kAnExpMaxEntries) t.n_hi = (int)hi;
+    return t;
+}
+
 // A warp per row, the row and its float Softmax in registers.
 template <int NITER>
 __global__ void __launch_bounds__(kAnThreads)
 analyze_softmax_kernel(const int32_t* __restrict__ scores, int64_t rows, int n, double in_scale, const __grid_constant__ AnSoftmax a,
-                       int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter, double* __restrict__ partials)
+                       int n_cand, const AnExp et, double* __restrict__ sums, unsigned* __restrict__ counter,
+                       double* __restrict__ partials)
 {
+    extern __shared__ __align__(16) double exp_lo[];                     // 2^shift low entries, then n_hi high ones
+    double* exp_hi = exp_lo + (1 << et.shift);
     grid_dep_launch();
+    if (et.n_hi) {
+        for (int i = threadIdx.x; i < 1 << et.shift; i += kAnThreads) exp_lo[i] = exp(-(double)i * in_scale);
+        for (int i = threadIdx.x; i < et.n_hi; i += kAnThreads) exp_hi[i] = exp(-((double)i * (double)(1 << et.shift)) * in_scale);
+        __syncthreads();
+    }
     grid_dep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t warp = (int64_t)blockIdx.x * (kAnThreads >> 5) + (threadIdx.x >> 5);
@@ -135,7 +164,13 @@ analyze_softmax_kernel(const int32_t* __restrict__ scores, int64_t rows, int n, 
         for (int k = 0; k < NITER; ++k) {
             X[k] = 0.0;
             if (k < iters) {                                             // uniform
-                if (lane + 32 * k < n) X[k] = exp(fma(an_to_double(v[k]), in_scale, -zmax));
+                if (et.n_hi) {
+                    // kNoScore is at a distance of 2^30 and more from every maximum: past the tables' range
+                    const unsigned d = (unsigned)mx - (unsigned)v[k];
+                    if ((d >> et.shift) < (unsigned)et.n_hi) X[k] = exp_hi[d >> et.shift] * exp_lo[d & ((1u << et.shift) - 1u)];
+                } else if (lane + 32 * k < n) {
+                    X[k] = exp(fma(an_to_double(v[k]), in_scale, -zmax));
+                }
                 den += X[k];
             }
         }
@@ -178,24 +213,62 @@ __device__ __forceinline__ int an_gelu(int x, const GeluDev& c)
     }
 }
 
+// What an input code contributes to every sum: X^2 and (X - Q_i)^2.
+struct AnGeluTerm {
+    double x2, e2[3];
+};
+static_assert(sizeof(AnGeluTerm) == 32, "one 32-byte sector per code");
+
+__device__ __forceinline__ AnGeluTerm an_gelu_term(int x, double in_scale, double out_scale, int out_zp, const AnGelu& a, int n_cand)
+{
+    const double v = an_to_double(x) * in_scale;
+    const double X = 0.5 * v * (1.0 + erf(v * 0.70710678118654752440));
+    AnGeluTerm t;
+    t.x2 = X * X;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        t.e2[i] = 0.0;
+        if (i < n_cand) {
+            const double d = X - an_to_double(an_gelu(x, a.c[i]) - out_zp) * out_scale;
+            t.e2[i] = d * d;
+        }
+    }
+    return t;
+}
+
+// Layers of kAnGeluTableMin elements and more: the terms of all 2^16 codes are tabulated first (2 MB, L2-resident) and an
+// element then costs one 32-byte read and four additions instead of an fp64 erf and three integer functions
+// (2.4 M elements: 54 us evaluated).  Below, the table would cost more than it saves.
+constexpr int64_t kAnGeluTableMin = 1 << 18;
+
+__global__ void __launch_bounds__(kAnThreads)
+analyze_gelu_terms_kernel(AnGeluTerm* __restrict__ table, double in_scale, double out_scale, int out_zp,
+                          const __grid_constant__ AnGelu a, int n_cand)
+{
+    grid_dep_launch();
+    const int i = blockIdx.x * kAnThreads + threadIdx.x;
+    const AnGeluTerm t = an_gelu_term(i - 32768, in_scale, out_scale, out_zp, a, n_cand);
+    grid_dep_wait();                                                     // the previous layer may still be reading the table
+    table[i] = t;
+}
+
 __global__ void __launch_bounds__(kAnThreads)
 analyze_gelu_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, double out_scale, int out_zp,
-                    const __grid_constant__ AnGelu a, int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter,
-                    double* __restrict__ partials)
+                    const __grid_constant__ AnGelu a, int n_cand, const AnGeluTerm* table, double* __restrict__ sums,
+                    unsigned* __restrict__ counter, double* __restrict__ partials)
 {
     grid_dep_launch();
     grid_dep_wait();
     double x2 = 0.0, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
     auto element = [&](int xi) {
-        const double v = an_to_double(xi) * in_scale;
-        const double X = 0.5 * v * (1.0 + erf(v * 0.70710678118654752440));
-        x2 = fma(X, X, x2);
-#pragma unroll
-        for (int i = 0; i < kAnMaxCand; ++i) {
-            if (i < n_cand) {
-                const double d = X - an_to_double(an_gelu(xi, a.c[i]) - out_zp) * out_scale;
-                e2[i] = fma(d, d, e2[i]);
-            }
+        if (table && xi >= -32768 && xi < 32768) {
+            // one 256-bit load per element, cached in L1: calibration activations fall on a few thousand codes
+            double t0, t1, t2, t3;
+            asm("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(t0), "=d"(t1), "=d"(t2), "=d"(t3) : "l"(table + 32768 + xi));
+            x2 += t0; e2[0] += t1; e2[1] += t2; e2[2] += t3;
+        } else {
+            const AnGeluTerm t = an_gelu_term(xi, in_scale, out_scale, out_zp, a, n_cand);
+            x2 += t.x2; e2[0] += t.e2[0]; e2[1] += t.e2[1]; e2[2] += t.e2[2];
         }
     };
     const int64_t nvec = n >> 2, stride = (int64_t)gridDim.x * kAnThreads, first = (int64_t)blockIdx.x * kAnThreads + threadIdx.x;
@@ -212,27 +285,64 @@ analyze_gelu_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, d
 // ------------------------------------------------------------------------------------------------ LayerNorm
 struct AnLayerNorm {
     int variant[kAnMaxCand];
+    bool same_out[kAnMaxCand];         // reads its input and requantises as the candidate before it
     RequantDev out[kAnMaxCand];
 };
 
+// The layer's parameters: by value in the launch up to MAXD channels (a copy to the device in front of every launch would
+// cost the stream more than a small layer's kernel), in device memory for wider layers.
+template <int MAXD>
+struct AnLnParams {
+    float4 gamma[MAXD / 4], beta[MAXD / 4];
+    int4 gamma_q[MAXD / 4], beta_q[MAXD / 4];
+    __device__ __forceinline__ void get(int i, float4& g, float4& b, int4& gq, int4& bq) const
+    {
+        g = gamma[i]; b = beta[i]; gq = gamma_q[i]; bq = beta_q[i];
+    }
+};
+template <>
+struct AnLnParams<0> {
+    const float4 *gamma, *beta;
+    const int4 *gamma_q, *beta_q;
+    __device__ __forceinline__ void get(int i, float4& g, float4& b, int4& gq, int4& bq) const
+    {
+        g = __ldg(gamma + i); b = __ldg(beta + i); gq = __ldg(gamma_q + i); bq = __ldg(beta_q + i);
+    }
+};
+constexpr int kAnLnBytesPerChannel = 24;                                 // shared memory: two doubles, two ints
+
 // A warp per row, under two readings of its input: index 0 plain, 1 with the power-of-two factors.  The row is read twice (the
-// second time from L1); the float parameters wait in shared memory as doubles.
+// second time from L1); the parameters wait in shared memory.  Bound by latency at calibration sizes (a few rows per warp).
+template <int MAXD>
 __global__ void __launch_bounds__(kAnThreads)
-analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, const float* __restrict__ gamma,
-                         const float* __restrict__ beta, const int32_t* __restrict__ gamma_q, const int32_t* __restrict__ beta_q,
+analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, const __grid_constant__ AnLnParams<MAXD> prm,
                          const uint8_t* __restrict__ ptf, double out_scale, int out_zp, const __grid_constant__ AnLayerNorm a,
                          int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter, double* __restrict__ partials)
 {
-    extern __shared__ __align__(16) double gb[];                         // gamma[D], beta[D]
-    grid_dep_launch();
-    grid_dep_wait();
-    for (int i = threadIdx.x; i < D; i += kAnThreads) { gb[i] = (double)__ldg(gamma + i); gb[D + i] = (double)__ldg(beta + i); }
-    __syncthreads();
+    extern __shared__ __align__(16) double2 gb[];                        // (gamma, beta) [D], then (gamma_q, beta_q) [D]
+    int2* gbq = reinterpret_cast<int2*>(gb + D);
     const int lane = threadIdx.x & 31, words = D >> 2;
+    grid_dep_launch();
+    if (MAXD == 0) grid_dep_wait();                                      // the parameters were copied to the device just before
+    // Read through a generic pointer the compiler cannot trace back: as constant-bank loads with an address per lane these
+    // reads go one address after the other, each a miss (10 us for 384 channels).
+    const AnLnParams<MAXD>* pp = &prm;
+    asm volatile("" : "+l"(pp));
+    for (int i = threadIdx.x; i < words; i += kAnThreads) {
+        float4 g, b;
+        int4 gq, bq;
+        pp->get(i, g, b, gq, bq);
+        gb[4 * i] = make_double2(g.x, b.x); gb[4 * i + 1] = make_double2(g.y, b.y);
+        gb[4 * i + 2] = make_double2(g.z, b.z); gb[4 * i + 3] = make_double2(g.w, b.w);
+        gbq[4 * i] = make_int2(gq.x, bq.x); gbq[4 * i + 1] = make_int2(gq.y, bq.y);
+        gbq[4 * i + 2] = make_int2(gq.z, bq.z); gbq[4 * i + 3] = make_int2(gq.w, bq.w);
+    }
+    __syncthreads();
+    if (MAXD != 0) grid_dep_wait();
     const int64_t warp = (int64_t)blockIdx.x * (kAnThreads >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (kAnThreads >> 5);
-    bool any_plain = false, any_ptf = false;
-    for (int i = 0; i < n_cand; ++i) { any_ptf |= a.variant[i] == IPTQ_LN_PTF; any_plain |= a.variant[i] != IPTQ_LN_PTF; }
+    bool any[2] = {false, false};
+    for (int i = 0; i < n_cand; ++i) any[a.variant[i] == IPTQ_LN_PTF] = true;
     double x2[2] = {0.0, 0.0}, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
     for (int64_t row = warp; row < rows; row += nwarps) {
         const int* xr = reinterpret_cast<const int*>(x + row * D);
@@ -240,11 +350,11 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
         unsigned s2[2] = {0, 0};
         for (int wi = lane; wi < words; wi += 32) {
             const int w = __ldg(xr + wi);
-            if (any_plain) {
+            if (any[0]) {
                 s1[0] = __dp4a(w, 0x01010101, s1[0]);
                 s2[0] = (unsigned)__dp4a(w, w, (int)s2[0]);
             }
-            if (any_ptf) {
+            if (any[1]) {
                 const unsigned sh = __ldg(reinterpret_cast<const unsigned*>(ptf) + wi);
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -255,51 +365,73 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
             }
         }
         double mu[2], inv_sd[2];
+        int f4[kAnMaxCand];
         long long F[kAnMaxCand];
+        bool same[kAnMaxCand];           // the candidate's integers in this row are those of the candidate before it
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             s1[p] = __reduce_add_sync(kAllLanes, s1[p]);
             s2[p] = __reduce_add_sync(kAllLanes, s2[p]);
+        }
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            if (!any[p]) continue;
             const long long V = (long long)D * (long long)s2[p] - (long long)s1[p] * (long long)s1[p];    // D^2 var
             mu[p] = (double)s1[p] / (double)D;
-            inv_sd[p] = V > 0 ? (double)D / sqrt((double)V) : 0.0;       // a constant row gives beta
+            inv_sd[p] = V > 0 ? (double)D * rsqrt((double)V) : 0.0;      // a constant row gives beta
+            const unsigned long long rt = ln_isqrt((unsigned long long)V, IPTQ_LN_NEWTON);
+            const long long Fn = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;
+            // the fixed steps of LN_SHIFT can end elsewhere only where V + 1 is a perfect square
+            const bool odd = (rt + 1) * (rt + 1) == (unsigned long long)V + 1;
 #pragma unroll
             for (int i = 0; i < kAnMaxCand; ++i) {
                 if (i < n_cand && (a.variant[i] == IPTQ_LN_PTF) == (p == 1)) {
-                    const unsigned long long rt = ln_isqrt((unsigned long long)V, a.variant[i]);
-                    F[i] = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;
+                    F[i] = Fn;
+                    if (a.variant[i] == IPTQ_LN_SHIFT && odd) {
+                        const unsigned long long r = ln_isqrt((unsigned long long)V, IPTQ_LN_SHIFT);
+                        F[i] = r ? (long long)floor_div_f64(1099511627776.0, (double)r) : 0;
+                    }
+                    f4[i] = F[i] < (1ll << 29) ? (int)(F[i] << 2) : 0;   // then (u F) >> 30 = hi32(u 4F)
                 }
             }
         }
+#pragma unroll
+        for (int i = 0; i < kAnMaxCand; ++i)
+            same[i] = i > 0 && i < n_cand && a.same_out[i] && F[i] == F[i - 1];
+        double er[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
         for (int wi = lane; wi < words; wi += 32) {
             const unsigned w = (unsigned)__ldg(xr + wi);
-            const unsigned sh = any_ptf ? __ldg(reinterpret_cast<const unsigned*>(ptf) + wi) : 0u;
-            const int4 g4 = __ldg(reinterpret_cast<const int4*>(gamma_q) + wi), b4 = __ldg(reinterpret_cast<const int4*>(beta_q) + wi);
-            const int gq[4] = {g4.x, g4.y, g4.z, g4.w}, bq[4] = {b4.x, b4.y, b4.z, b4.w};
+            const unsigned sh = any[1] ? __ldg(reinterpret_cast<const unsigned*>(ptf) + wi) : 0u;
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 const int xv[2] = {(int)(int8_t)(w >> (8 * t)), ((int)(int8_t)(w >> (8 * t))) << ((sh >> (8 * t)) & 3)};
-                const double ga = gb[4 * wi + t], be = gb[D + 4 * wi + t];
+                const double2 fp = gb[4 * wi + t];
+                const int2 qp = gbq[4 * wi + t];
                 double X[2] = {0.0, 0.0};
 #pragma unroll
                 for (int p = 0; p < 2; ++p) {
-                    if (p == 0 ? any_plain : any_ptf) {
-                        X[p] = fma((an_to_double(xv[p]) - mu[p]) * inv_sd[p], ga, be);
+                    if (any[p]) {
+                        X[p] = fma((an_to_double(xv[p]) - mu[p]) * inv_sd[p], fp.x, fp.y);
                         x2[p] = fma(X[p], X[p], x2[p]);
                     }
                 }
 #pragma unroll
                 for (int i = 0; i < kAnMaxCand; ++i) {
-                    if (i < n_cand) {
+                    if (i < n_cand && !same[i]) {
                         const int p = a.variant[i] == IPTQ_LN_PTF ? 1 : 0;
                         const int u = D * (p ? xv[1] : xv[0]) - (p ? s1[1] : s1[0]);
-                        const int nq = (int)(((long long)u * F[i]) >> 30);
-                        const int o = requant_full(nq * gq[t] + bq[t], a.out[i]);
+                        const int nq = f4[i] ? __mulhi(u, f4[i]) : (int)(((long long)u * F[i]) >> 30);
+                        const int o = requant_full(nq * qp.x + qp.y, a.out[i]);
                         const double d = (p ? X[1] : X[0]) - an_to_double(o - out_zp) * out_scale;
-                        e2[i] = fma(d, d, e2[i]);
+                        er[i] = fma(d, d, er[i]);
                     }
                 }
             }
+        }
+#pragma unroll
+        for (int i = 0; i < kAnMaxCand; ++i) {
+            if (i > 0 && i < n_cand && same[i]) er[i] = er[i - 1];
+            e2[i] += er[i];
         }
     }
     double xs[kAnMaxCand];
@@ -308,9 +440,9 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
     an_finish(xs, e2, n_cand, sums, counter, partials);
 }
 
-static int an_grid(int64_t blocks)
+static int an_grid(int64_t blocks, int per_sm = 4)
 {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, std::min<int64_t>((int64_t)sm_count() * 4, kAnMaxBlocks)));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, std::min<int64_t>((int64_t)sm_count() * per_sm, kAnMaxBlocks)));
 }
 
 static int an_args_ok(const void* consts, int n_cand, const void* sums, const void* work)
@@ -349,10 +481,11 @@ int iptq_analyze_softmax(const int32_t* scores, int64_t rows, int row_len, doubl
     }
     unsigned* counter = static_cast<unsigned*>(work);
     double* partials = reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256);
+    const AnExp et = an_exp(in_scale);
     const int grid = an_grid((rows + 7) / 8), it = (row_len + 31) / 32;
 #define IPTQ_AN_SM(NI)                                                                                                    \
-    launch_kernel(analyze_softmax_kernel<NI>, grid, kAnThreads, 0, stream, scores, rows, row_len, in_scale, a, n_candidates, \
-                  sums, counter, partials)
+    launch_kernel(analyze_softmax_kernel<NI>, grid, kAnThreads, et.n_hi ? 8 * ((size_t)et.n_hi + (1u << et.shift)) : 0, stream, \
+                  scores, rows, row_len, in_scale, a, n_candidates, et, sums, counter, partials)
     if (it <= 2) IPTQ_AN_SM(2);
     else if (it <= 4) IPTQ_AN_SM(4);
     else if (it <= 5) IPTQ_AN_SM(5);
@@ -370,7 +503,7 @@ int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_s
 {
     int rc = an_args_ok(consts, n_candidates, sums, work);
     if (rc != IPTQ_OK) return rc;
-    if (n < 0) return IPTQ_ERR_SHAPE;
+    if (n < 0 || n_candidates > 3) return IPTQ_ERR_SHAPE;
     if (!(in_scale > 0.0) || !(out_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
     if (n > 0 && !x) return IPTQ_ERR_NULL;
     if (!aligned16(x)) return IPTQ_ERR_ALIGN;
@@ -381,9 +514,17 @@ int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_s
         if ((rc = check_requant(&consts[i].out)) != IPTQ_OK) return rc;
         a.c[i] = to_dev(consts[i]);
     }
-    launch_kernel(analyze_gelu_kernel, an_grid((n / 4 + kAnThreads - 1) / kAnThreads), kAnThreads, 0, stream, x, n, in_scale,
-                  out_scale, out_zp, a, n_candidates, sums, static_cast<unsigned*>(work),
-                  reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256));
+    unsigned* counter = static_cast<unsigned*>(work);
+    double* partials = reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256);
+    AnGeluTerm* table = nullptr;
+    if (n >= kAnGeluTableMin) {
+        table = reinterpret_cast<AnGeluTerm*>(static_cast<uint8_t*>(work) + kAnPartialBytes);
+        launch_kernel(analyze_gelu_terms_kernel, 65536 / kAnThreads, kAnThreads, 0, stream, table, in_scale, out_scale, out_zp, a,
+                      n_candidates);
+        note_launch();
+    }
+    launch_kernel(analyze_gelu_kernel, an_grid((n / 4 + kAnThreads - 1) / kAnThreads, table ? 6 : 4), kAnThreads, 0, stream, x, n, in_scale,
+                  out_scale, out_zp, a, n_candidates, table, sums, counter, partials);
     note_launch();
     return last_launch_status();
 }
@@ -398,7 +539,7 @@ int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* 
     if (rows < 0 || dim < 4 || dim > 3072 || (dim & 3)) return IPTQ_ERR_SHAPE;
     if (!(out_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
     if (!gamma || !beta || !gamma_q || !beta_q || (rows > 0 && !x)) return IPTQ_ERR_NULL;
-    if (!aligned16(x) || !aligned16(gamma_q) || !aligned16(beta_q) || (reinterpret_cast<uintptr_t>(ptf_shift) & 3u)) return IPTQ_ERR_ALIGN;
+    if (!aligned16(x) || (reinterpret_cast<uintptr_t>(ptf_shift) & 3u)) return IPTQ_ERR_ALIGN;
     AnLayerNorm a{};
     for (int i = 0; i < n_candidates; ++i) {
         if (consts[i].dim != dim) return IPTQ_ERR_SHAPE;
@@ -407,13 +548,41 @@ int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* 
         if ((rc = check_requant(&consts[i].out)) != IPTQ_OK) return rc;
         a.variant[i] = consts[i].variant;
         a.out[i] = to_dev(consts[i].out);
+        a.same_out[i] = i > 0 && (a.variant[i] == IPTQ_LN_PTF) == (a.variant[i - 1] == IPTQ_LN_PTF) &&
+                        memcmp(&consts[i].out, &consts[i - 1].out, sizeof(iptq_requant)) == 0;
     }
-    // 16 bytes per channel beside the static shared memory: wide rows pass the default limit of 48 KB
-    if (dim > 2048 && cudaFuncSetAttribute(analyze_layernorm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 3072) != cudaSuccess)
-        return IPTQ_ERR_CUDA;
-    launch_kernel(analyze_layernorm_kernel, an_grid((rows + 7) / 8), kAnThreads, (size_t)16 * dim, stream, x, rows, dim, gamma,
-                  beta, gamma_q, beta_q, ptf_shift, out_scale, out_zp, a, n_candidates, sums, static_cast<unsigned*>(work),
-                  reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256));
+    unsigned* counter = static_cast<unsigned*>(work);
+    double* partials = reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256);
+    const int grid = an_grid((rows + 7) / 8);
+    const size_t smem = (size_t)kAnLnBytesPerChannel * dim, bytes = (size_t)dim * 4;
+    auto by_value = [&](auto& prm, auto kern) {
+        memcpy(prm.gamma, gamma, bytes); memcpy(prm.beta, beta, bytes);
+        memcpy(prm.gamma_q, gamma_q, bytes); memcpy(prm.beta_q, beta_q, bytes);
+        launch_kernel(kern, grid, kAnThreads, smem, stream, x, rows, dim, prm, ptf_shift, out_scale, out_zp, a, n_candidates, sums,
+                      counter, partials);
+    };
+    if (dim <= 256) {
+        AnLnParams<256> prm;
+        by_value(prm, analyze_layernorm_kernel<256>);
+    } else if (dim <= 512) {
+        AnLnParams<512> prm;
+        by_value(prm, analyze_layernorm_kernel<512>);
+    } else if (dim <= 1024) {
+        AnLnParams<1024> prm;
+        by_value(prm, analyze_layernorm_kernel<1024>);
+    } else {
+        // where the GELU terms of another layer would be: the copies come after every earlier launch that uses the scratch
+        uint8_t* dst = static_cast<uint8_t*>(work) + kAnPartialBytes;
+        const void* src[4] = {gamma, beta, gamma_q, beta_q};
+        for (int i = 0; i < 4; ++i)
+            if (cudaMemcpyAsync(dst + (size_t)i * 3072 * 4, src[i], bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return IPTQ_ERR_CUDA;
+        AnLnParams<0> prm{reinterpret_cast<const float4*>(dst), reinterpret_cast<const float4*>(dst + 3072 * 4),
+                          reinterpret_cast<const int4*>(dst + 2 * 3072 * 4), reinterpret_cast<const int4*>(dst + 3 * 3072 * 4)};
+        if (cudaFuncSetAttribute(analyze_layernorm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnLnBytesPerChannel * 3072) != cudaSuccess)
+            return IPTQ_ERR_CUDA;
+        launch_kernel(analyze_layernorm_kernel<0>, grid, kAnThreads, smem, stream, x, rows, dim, prm, ptf_shift, out_scale, out_zp, a,
+                      n_candidates, sums, counter, partials);
+    }
     note_launch();
     return last_launch_status();
 }

@@ -354,30 +354,24 @@ PyObject* analyze_layernorm(PyObject* const* a, Py_ssize_t)
     const int dim = (int)x.size(1), zp = (int)integer(a[4]), bits = (int)integer(a[5]);
     const float *gamma = host_floats(a[1], dim), *beta = host_floats(a[2], dim);
     const double out_scale = real(a[3]);
-    // the float and the integer parameters of the layer go to the device in one copy
-    const size_t part = ((size_t)dim * 4 + 15) & ~(size_t)15;
-    std::vector<uint8_t> host(4 * part);
-    memcpy(host.data(), gamma, (size_t)dim * 4);
-    memcpy(host.data() + part, beta, (size_t)dim * 4);
-    int32_t *gq = reinterpret_cast<int32_t*>(host.data() + 2 * part), *bq = reinterpret_cast<int32_t*>(host.data() + 3 * part);
+    std::vector<int32_t> q((size_t)2 * dim);
+    int32_t *gq = q.data(), *bq = q.data() + dim;
     iptq_ln_consts c[IPTQ_ANALYZE_MAX_CANDIDATES];
     int ids[IPTQ_ANALYZE_MAX_CANDIDATES];
     const int n = prepare_candidates(a[6], c, ids, [&](int v, iptq_ln_consts* out) {
         if (v == IPTQ_LN_PTF && a[7] == Py_None) return (int)IPTQ_ERR_NULL;      // a candidate for inputs with such factors alone
+        if (out != c && v >= IPTQ_LN_SHIFT && v <= IPTQ_LN_PTF) {       // the variant is all that differs between the candidates
+            *out = c[0];
+            out->variant = v;
+            return (int)IPTQ_OK;
+        }
         check(api.layernorm_prepare(dim, gamma, beta, out_scale, zp, bits, (iptq_ln_variant)v, gq, bq, out), "iptq_layernorm_prepare");
         return (int)IPTQ_OK;
     });
-    if (n) {
-        at::Tensor d = at::detail::empty_cuda({(int64_t)host.size()}, at::kByte, x.device(), std::nullopt);
-        const cudaStream_t st = stream();
-        if (cudaMemcpyAsync(d.data_ptr(), host.data(), host.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
-            check(IPTQ_ERR_CUDA, "cudaMemcpyAsync");
-        uint8_t* p = static_cast<uint8_t*>(d.data_ptr());
-        check(api.analyze_layernorm(static_cast<const int8_t*>(x.data_ptr()), x.size(0), dim, reinterpret_cast<float*>(p),
-                                    reinterpret_cast<float*>(p + part), reinterpret_cast<int32_t*>(p + 2 * part),
-                                    reinterpret_cast<int32_t*>(p + 3 * part), dev<uint8_t>(a[7]), out_scale, zp, c, n,
-                                    static_cast<double*>(address(a[8])), address(a[9]), st), "iptq_analyze_layernorm");
-    }
+    if (n)
+        check(api.analyze_layernorm(static_cast<const int8_t*>(x.data_ptr()), x.size(0), dim, gamma, beta, gq, bq, dev<uint8_t>(a[7]),
+                                    out_scale, zp, c, n, static_cast<double*>(address(a[8])), address(a[9]), stream()),
+              "iptq_analyze_layernorm");
     return candidate_list(IPTQ_LAYER_LAYERNORM, ids, n, x.size(0), dim);
 }
 

@@ -379,17 +379,16 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
             const long long V = (long long)D * (long long)s2[p] - (long long)s1[p] * (long long)s1[p];    // D^2 var
             mu[p] = (double)s1[p] / (double)D;
             inv_sd[p] = V > 0 ? (double)D * rsqrt((double)V) : 0.0;      // a constant row gives beta
-            const unsigned long long rt = ln_isqrt((unsigned long long)V, IPTQ_LN_NEWTON);
-            const long long Fn = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;
+            const double rt = ln_isqrt((double)V, IPTQ_LN_NEWTON);
+            const long long Fn = (long long)ln_reciprocal(rt);
             // the fixed steps of LN_SHIFT can end elsewhere only where V + 1 is a perfect square
-            const bool odd = (rt + 1) * (rt + 1) == (unsigned long long)V + 1;
+            const bool odd = rt > 0.0 && (rt + 1.0) * (rt + 1.0) == (double)V + 1.0;
 #pragma unroll
             for (int i = 0; i < kAnMaxCand; ++i) {
                 if (i < n_cand && (a.variant[i] == IPTQ_LN_PTF) == (p == 1)) {
                     F[i] = Fn;
                     if (a.variant[i] == IPTQ_LN_SHIFT && odd) {
-                        const unsigned long long r = ln_isqrt((unsigned long long)V, IPTQ_LN_SHIFT);
-                        F[i] = r ? (long long)floor_div_f64(1099511627776.0, (double)r) : 0;
+                        F[i] = (long long)ln_reciprocal(ln_isqrt((double)V, IPTQ_LN_SHIFT));
                     }
                     f4[i] = F[i] < (1ll << 29) ? (int)(F[i] << 2) : 0;   // then (u F) >> 30 = hi32(u 4F)
                 }

@@ -107,7 +107,7 @@ static int encoder_block_run(const int8_t* x, int8_t* y, const iptq_block_params
         if ((rc = unpack_int4_multi_launch(srcs, dsts, ns, 4, stream)) != IPTQ_OK) return rc;   // one launch for the four matrices
     }
 
-    if ((rc = layernorm_launch(x, h1, T, D, p->ln1_gamma, p->ln1_beta, p->ln1_ptf, p->ln1, stream)) != IPTQ_OK) return rc;
+    if ((rc = layernorm_launch(LnArgs{x, p->ln1_gamma, p->ln1_beta, p->ln1_ptf, p->ln1}, h1, T, D, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
     const int ab = p->act_bits ? p->act_bits : 8;            // width of the QKV / proj / FC2 outputs
     if (ab < 4 || ab > 8) return IPTQ_ERR_BITS;
@@ -122,7 +122,7 @@ static int encoder_block_run(const int8_t* x, int8_t* y, const iptq_block_params
     LinearArgs lp{att, wp, p->b_proj, p->m_proj, p->s_proj, p->proj_zp, x, p->res1_rq, nullptr, x1, T, D, D, status, ab};
     if ((rc = linear_launch(lp, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
-    if ((rc = layernorm_launch(x1, h2, T, D, p->ln2_gamma, p->ln2_beta, p->ln2_ptf, p->ln2, stream)) != IPTQ_OK) return rc;
+    if ((rc = layernorm_launch(LnArgs{x1, p->ln2_gamma, p->ln2_beta, p->ln2_ptf, p->ln2}, h2, T, D, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
     LinearArgs l1{h2, w1, p->b_fc1, p->m_fc1, p->s_fc1, 0, nullptr, nullptr, p->gelu, hid, T, Dh, D, status};
     if ((rc = linear_launch(l1, stream)) != IPTQ_OK) return rc;

@@ -277,41 +277,47 @@ __device__ __forceinline__ int gelu_core(int x, const GeluDev& c)
 }
 
 // ---- integer statistics of the LayerNorm
-__device__ __forceinline__ unsigned long long isqrt_floor(unsigned long long V)
-{
-    // V >= 1.  Estimate from the hardware reciprocal square root (about 22 good bits), then walk to the exact
-    // floor with the remainder e = V - s^2: one or two steps for the 44-bit values of this kernel.
-    const double vd = (double)(long long)V;
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(vd));
-    long long s = (long long)(vd * y);
-    long long e = (long long)V - s * s;
-    while (e < 0) { --s; e += 2 * s + 1; }
-    while (e > 2 * s) { e -= 2 * s + 1; ++s; }
-    return (unsigned long long)s;
-}
-
 // floor(a / b) for integers 0 <= a < 2^53, 1 <= b with a / b * b <= 2^53: the correctly rounded fp64 quotient of
 // a non-integer a / b lies at least 1 / b below the next integer, i.e. 2^-53 relatively away whenever the
 // quotient times b stays below 2^53, so truncation gives the exact floor.
 __device__ __forceinline__ double floor_div_f64(double a, double b) { return floor(a / b); }
 
-__device__ __forceinline__ unsigned long long ln_isqrt(unsigned long long V, int variant)
+// D * std of a row: the integer square root of V = D^2 var (an integer below 2^46) as the variant defines it, in fp64.
+// Hardware estimate of 1 / sqrt(V) (20 bits and more), one Newton step (40 bits of a 23-bit root: off by far less than
+// one), and the exact remainder e = V - s^2, which says whether the truncated root is one too large or too small.
+__device__ __forceinline__ double ln_isqrt(double V, int variant)
 {
-    if (V == 0) return 0;
-    const unsigned long long s = isqrt_floor(V);
-    if (variant != IPTQ_LN_SHIFT) return s;
-    // Fixed 10 steps of r <- (r + V / r) >> 1 from 2^ceil(bitlen(V) / 2), no convergence test.  From a start
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(V));
+    double s = V * y;
+    s = floor(fma(fma(-s, s, V), 0.5 * y, s));
+    double e = fma(-s, s, V);
+    if (e < 0.0) { s -= 1.0; e = fma(-s, s, V); }
+    if (e > 2.0 * s) { s += 1.0; e = fma(-s, s, V); }
+    if (V == 0.0) return 0.0;
+    // LN_SHIFT: fixed 10 steps of r <- (r + V / r) >> 1 from 2^ceil(bitlen(V) / 2), no convergence test.  From a start
     // within a factor 2 of sqrt(V) the recurrence reaches floor(sqrt V) in at most 7 steps and then stays there,
-    // except when V + 1 is a perfect square, where it alternates between s and s + 1: only then is the
-    // recurrence actually run (in fp64, every intermediate is an exact integer below 2^53).
-    if ((s + 1) * (s + 1) != V + 1) return s;
+    // except when V + 1 is a perfect square, (s + 1)^2 = V + 1, where it alternates between s and s + 1: only then is
+    // the recurrence actually run (every intermediate is an exact integer below 2^53).
+    if (variant != IPTQ_LN_SHIFT || e != 2.0 * s) return s;
     const int w = 64 - __clzll((long long)V);
     double r = (double)(1ull << ((w + 1) >> 1));
-    const double Vd = (double)V;
 #pragma unroll 1
-    for (int it = 0; it < 10; ++it) r = floor((r + floor_div_f64(Vd, r)) * 0.5);
-    return (unsigned long long)r;
+    for (int it = 0; it < 10; ++it) r = floor((r + floor_div_f64(V, r)) * 0.5);
+    return r;
+}
+
+// F = floor(2^40 / rt) for an integer rt >= 1 (0 for rt = 0): hardware estimate of 1 / rt, one Newton step, exact remainder.
+__device__ __forceinline__ double ln_reciprocal(double rt)
+{
+    double z;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(rt));
+    z = fma(fma(-rt, z, 1.0), z, z);
+    double q = floor(1099511627776.0 * z);
+    const double e = fma(-q, rt, 1099511627776.0);
+    if (e < 0.0) q -= 1.0;
+    else if (e >= rt) q += 1.0;
+    return rt > 0.0 ? q : 0.0;
 }
 
 __device__ __forceinline__ unsigned pack4_s8(int a, int b, int c, int d)

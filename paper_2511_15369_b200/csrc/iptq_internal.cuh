@@ -26,9 +26,15 @@ int unpack_int4_launch(const void* packed, int8_t* out, int64_t n_elems, cudaStr
 int unpack_int4_multi_launch(const void* const* packed, int8_t* const* out, const int64_t* n_elems, int count,
                              cudaStream_t st);
 
-// ---------------------------------------------------------------- LayerNorm (nonlinear.cu)
-int layernorm_launch(const int8_t* x, int8_t* y, int64_t rows, int dim, const int32_t* gq, const int32_t* bq,
-                     const uint8_t* ptf, const iptq_ln_consts* consts, cudaStream_t st);
+// ---------------------------------------------------------------- LayerNorm (layernorm.cu)
+struct LnArgs {
+    const int8_t* x; const int32_t *gamma, *beta; const uint8_t* ptf;
+    const iptq_ln_consts* consts;
+    const int32_t* index = nullptr;    // source rows: output row i is the LayerNorm of the concatenated rows index[i * parts + p] of
+    int parts = 1;                     // x (each dim / parts channels, negative: zeros); null: of row i
+};
+int layernorm_check(const LnArgs& a, const int8_t* y, int64_t rows, int dim);
+int layernorm_launch(const LnArgs& a, int8_t* y, int64_t rows, int dim, cudaStream_t st);
 
 // ---------------------------------------------------------------- fused attention (attention.cu)
 // Strided q/k/v so that the encoder block can read heads straight out of the fused QKV activation.

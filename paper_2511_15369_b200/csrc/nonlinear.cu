@@ -1,4 +1,4 @@
-// Stand-alone integer Softmax / GELU / LayerNorm kernels (row- and element-wise, HBM/ALU bound).
+// Stand-alone integer Softmax / GELU kernels (row- and element-wise, HBM/ALU bound).
 #include <climits>
 #include <type_traits>
 
@@ -322,354 +322,6 @@ softmax_table_kernel(uint16_t* __restrict__ table, int n, int n_pad, const ExpDe
 // and visible, so a later kernel that reads the table ahead of its own dependency wait cannot overtake the writer.
 __global__ void stream_fence_kernel() {}
 
-// ------------------------------------------------------------------------------------------------
-// LayerNorm: a warp takes a few rows at a time; the rows live in registers as packed int8 words (NW per lane).
-// ------------------------------------------------------------------------------------------------
-struct LnDev {
-    int variant, dim;
-    RequantDev out;
-};
-
-// One warp handles RW rows at a time.  The per-row scalar work (variance, integer square root, reciprocal) is the
-// long dependent chain of this kernel; lane r of the warp runs it for row r, so its cost is shared by RW rows.
-// EXACT: the row is exactly 32 * NW words, so no lane ever needs a bounds predicate.  ZPF: the output zero point is
-// folded into the rounding constant (c.out.rnd already holds rnd + (zp << shift), c.out.zp is 0).  PREFETCH: the rows
-// of a warp's next group are loaded before the current group is processed (pays off once a warp has several groups).
-template <int NW, int RW, bool PTF, bool SAT8, bool EXACT, bool ZPF, bool PREFETCH>
-__global__ void __launch_bounds__(256)
-layernorm_rows_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, int64_t rows,
-                      const int32_t* __restrict__ gamma_q, const int32_t* __restrict__ beta_q,
-                      const uint8_t* __restrict__ ptf, const LnDev c)
-{
-    const int lane = threadIdx.x & 31;
-    const int D = c.dim;
-    grid_dep_launch();
-    const int words = D >> 2;
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t groups = (rows + RW - 1) / RW;
-    // per-lane channel parameters stay in registers across rows when they fit
-    constexpr bool KEEP = NW <= 8;
-    int4 g[KEEP ? NW : 1], b[KEEP ? NW : 1];
-    unsigned sh[NW];
-#pragma unroll
-    for (int k = 0; k < NW; ++k) {
-        const int wi = lane + 32 * k;
-        sh[k] = 0;
-        if (EXACT || wi < words) {
-            if (KEEP) {
-                g[k] = __ldg(reinterpret_cast<const int4*>(gamma_q) + wi);
-                b[k] = __ldg(reinterpret_cast<const int4*>(beta_q) + wi);
-            }
-            if (PTF) sh[k] = __ldg(reinterpret_cast<const unsigned*>(ptf) + wi);
-        }
-    }
-    grid_dep_wait();                                // gamma / beta above are static; the rows come from the previous kernel
-    // the rows of the next group are fetched while the current group is processed
-    auto fetch = [&](int64_t grp, int (&dst)[RW][NW]) {
-        const int64_t row0 = grp * RW;
-#pragma unroll
-        for (int r = 0; r < RW; ++r) {
-            const bool live = grp < groups && row0 + r < rows;
-            const int* xr = reinterpret_cast<const int*>(x + (live ? row0 + r : 0) * D);
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                const int wi = lane + 32 * k;
-                dst[r][k] = (live && (EXACT || wi < words)) ? __ldcs(xr + wi) : 0;
-            }
-        }
-    };
-    int wn[PREFETCH ? RW : 1][PREFETCH ? NW : 1];
-    if constexpr (PREFETCH) fetch(warp, wn);
-    for (int64_t grp = warp; grp < groups; grp += nwarps) {
-        const int64_t row0 = grp * RW;
-        int w[RW][NW];
-        if constexpr (PREFETCH) {
-#pragma unroll
-            for (int r = 0; r < RW; ++r)
-#pragma unroll
-                for (int k = 0; k < NW; ++k) w[r][k] = wn[r][k];
-            fetch(grp + nwarps, wn);
-        } else {
-            fetch(grp, w);
-        }
-        int my_s1 = 0;
-        unsigned my_s2 = 0;
-#pragma unroll
-        for (int r = 0; r < RW; ++r) {
-            int s1 = 0;
-            unsigned s2 = 0;
-#pragma unroll
-            for (int k = 0; k < NW; ++k) {
-                if (!PTF) {
-                    s1 = __dp4a(w[r][k], 0x01010101, s1);
-                    s2 = (unsigned)__dp4a(w[r][k], w[r][k], (int)s2);
-                } else {
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const int xv = ((int)(int8_t)(w[r][k] >> (8 * t))) << ((sh[k] >> (8 * t)) & 3);
-                        s1 += xv;
-                        s2 += (unsigned)(xv * xv);
-                    }
-                }
-            }
-            s1 = __reduce_add_sync(kFull, s1);
-            s2 = __reduce_add_sync(kFull, s2);
-            if (lane == r) { my_s1 = s1; my_s2 = s2; }
-        }
-        // lane r: statistics of row r (the other lanes run the same instructions on zeros)
-        const long long V = (long long)D * (long long)my_s2 - (long long)my_s1 * (long long)my_s1;   // D^2 var, exact
-        const unsigned long long rt = ln_isqrt((unsigned long long)V, c.variant);                // D * std
-        const long long F = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;          // floor(2^40 / rt)
-        // (u F) >> 30 = hi32(u * 4F) when 4F fits in 32 bits (rows whose D * std exceeds 2^11: all but near-constant rows)
-        const int my_narrow = F < (1ll << 29);
-        const int my_F4 = (int)(F << 2);
-#pragma unroll
-        for (int r = 0; r < RW; ++r) {
-            if (row0 + r >= rows) break;                                        // warp-uniform
-            const int s1 = __shfl_sync(kFull, my_s1, r);
-            const int F4 = __shfl_sync(kFull, my_F4, r);
-            const bool narrow = __shfl_sync(kFull, my_narrow, r) != 0;
-            const long long Fr = narrow ? 0 : (((long long)__shfl_sync(kFull, (int)(F >> 32), r) << 32) |
-                                               (unsigned)__shfl_sync(kFull, (int)(unsigned)F, r));
-            int* yr = reinterpret_cast<int*>(y + (row0 + r) * D);
-            const int om = c.out.mult, ornd = c.out.rnd, osh = c.out.shift, ozp = c.out.zp;
-            auto emit = [&](auto narrow_c) {
-                constexpr bool NARROW = decltype(narrow_c)::value;
-                auto elem = [&](int xv, unsigned shw, int t, int gg, int bb) -> int {
-                    if (PTF) xv <<= ((shw >> (8 * t)) & 3);
-                    const int u = D * xv - s1;                                   // D (x - mean)
-                    const int nq = NARROW ? __mulhi(u, F4) : (int)(((long long)u * Fr) >> 30);   // (x - mean) / std, Q10
-                    int o = mad_hi(nq * gg + bb, om, ornd) >> osh;
-                    if (!ZPF) o += ozp;
-                    if (!SAT8) o = max(c.out.qmin, min(c.out.qmax, o));
-                    return o;
-                };
-#pragma unroll
-                for (int k = 0; k < NW; ++k) {
-                    const int wi = lane + 32 * k;
-                    if (EXACT || wi < words) {
-                        int4 gg, bb;
-                        if (KEEP) { gg = g[k]; bb = b[k]; }
-                        else {
-                            gg = __ldg(reinterpret_cast<const int4*>(gamma_q) + wi);
-                            bb = __ldg(reinterpret_cast<const int4*>(beta_q) + wi);
-                        }
-                        const unsigned wk = (unsigned)w[r][k];
-                        const int o0 = elem(sext_byte<0>(wk), sh[k], 0, gg.x, bb.x);
-                        const int o1 = elem(sext_byte<1>(wk), sh[k], 1, gg.y, bb.y);
-                        const int o2 = elem(sext_byte<2>(wk), sh[k], 2, gg.z, bb.z);
-                        const int o3 = elem(sext_byte<3>(wk), sh[k], 3, gg.w, bb.w);
-                        __stcs(yr + wi, SAT8 ? (int)pack4_sat_s8(o0, o1, o2, o3) : (int)pack4_s8(o0, o1, o2, o3));
-                    }
-                }
-            };
-            if (narrow) emit(std::true_type{});
-            else        emit(std::false_type{});
-        }
-    }
-}
-
-// Short rows (dim <= 128, dim % 16 == 0: the first Swin stage): LPR lanes share a row, so a warp step covers 32 / LPR
-// rows.  Lane q of a row takes words q, q + LPR, ... (WPL = dim / (4 LPR) words); row sums are xor-shuffles over the
-// LPR lanes, and every lane then runs the scalar part (variance, square root, reciprocal) of its own row, so the
-// hundred dependent instructions of that part are shared by 32 / LPR rows without any broadcast.  Two lanes per row
-// up to 96 channels (16 rows per scalar part: 96 channels 20.8 -> 19.5 us, 64 channels 17.4 -> 15.1 us on 200 k rows),
-// four at 128, where twelve more words per lane would spill.
-template <int LPR, int WPL, bool PTF, bool SAT8, bool ZPF>
-__global__ void __launch_bounds__(256, 4)
-layernorm_short_rows_kernel(const int8_t* __restrict__ x, int8_t* __restrict__ y, int64_t rows,
-                            const int32_t* __restrict__ gamma_q, const int32_t* __restrict__ beta_q,
-                            const uint8_t* __restrict__ ptf, const LnDev c)
-{
-    const int lane = threadIdx.x & 31;
-    constexpr int RPW = 32 / LPR;                             // rows per warp step
-    const int q = lane & (LPR - 1);                           // position inside the row's lanes
-    const int D = c.dim;                                      // = 16 * WPL
-    grid_dep_launch();
-    const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t steps = (rows + RPW - 1) / RPW;
-    // The per-channel parameters live in shared memory (the lanes of a row read consecutive addresses, the rows of a
-    // warp the same ones: no bank conflict).  In registers they are 48 per thread and halve the resident warps, and
-    // resident warps are what hides a row's chain of dependent steps (load, two reductions, square root, divide):
-    // 64 registers and four CTAs per SM instead of 98 and two took the 96-channel case from 25.0 to 20.8 us.
-    __shared__ int4 g[LPR * WPL], b[LPR * WPL];
-    unsigned sh[WPL];
-    for (int i = threadIdx.x; i < LPR * WPL; i += blockDim.x) {
-        g[i] = __ldg(reinterpret_cast<const int4*>(gamma_q) + i);
-        b[i] = __ldg(reinterpret_cast<const int4*>(beta_q) + i);
-    }
-#pragma unroll
-    for (int k = 0; k < WPL; ++k) sh[k] = PTF ? __ldg(reinterpret_cast<const unsigned*>(ptf) + q + LPR * k) : 0u;
-    __syncthreads();
-    grid_dep_wait();                                          // gamma / beta above are static; the rows come from the previous kernel
-    const int om = c.out.mult, ornd = c.out.rnd, osh = c.out.shift, ozp = c.out.zp;
-    for (int64_t step = warp; step < steps; step += nwarps) {
-        const int64_t row = step * RPW + lane / LPR;
-        const bool live = row < rows;
-        const int* xr = reinterpret_cast<const int*>(x + (live ? row : 0) * D);
-        int w[WPL];
-#pragma unroll
-        for (int k = 0; k < WPL; ++k) w[k] = live ? __ldcs(xr + q + LPR * k) : 0;
-        int s1 = 0;
-        unsigned s2 = 0;
-#pragma unroll
-        for (int k = 0; k < WPL; ++k) {
-            if (!PTF) {
-                s1 = __dp4a(w[k], 0x01010101, s1);
-                s2 = (unsigned)__dp4a(w[k], w[k], (int)s2);
-            } else {
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const int xv = ((int)(int8_t)(w[k] >> (8 * t))) << ((sh[k] >> (8 * t)) & 3);
-                    s1 += xv;
-                    s2 += (unsigned)(xv * xv);
-                }
-            }
-        }
-        s1 += __shfl_xor_sync(kFull, s1, 1); s2 += __shfl_xor_sync(kFull, s2, 1);
-        if (LPR == 4) { s1 += __shfl_xor_sync(kFull, s1, 2); s2 += __shfl_xor_sync(kFull, s2, 2); }
-        const long long V = (long long)D * (long long)s2 - (long long)s1 * (long long)s1;            // D^2 var, exact
-        const unsigned long long rt = ln_isqrt((unsigned long long)V, c.variant);                // D * std
-        const long long F = rt ? (long long)floor_div_f64(1099511627776.0, (double)rt) : 0;          // floor(2^40 / rt)
-        const bool narrow = F < (1ll << 29);                  // then (u F) >> 30 = hi32(u * 4F)
-        const int F4 = (int)(F << 2);
-        int out[WPL];
-#pragma unroll
-        for (int k = 0; k < WPL; ++k) {
-            const unsigned wk = (unsigned)w[k];
-            auto elem = [&](int xv, int t, int gg, int bb) -> int {
-                if (PTF) xv <<= ((sh[k] >> (8 * t)) & 3);
-                const int u = D * xv - s1;                                   // D (x - mean)
-                const int nq = narrow ? __mulhi(u, F4) : (int)(((long long)u * F) >> 30);   // (x - mean) / std, Q10
-                int o = mad_hi(nq * gg + bb, om, ornd) >> osh;
-                if (!ZPF) o += ozp;
-                if (!SAT8) o = max(c.out.qmin, min(c.out.qmax, o));
-                return o;
-            };
-            const int4 gk = g[q + LPR * k], bk = b[q + LPR * k];
-            const int o0 = elem(sext_byte<0>(wk), 0, gk.x, bk.x);
-            const int o1 = elem(sext_byte<1>(wk), 1, gk.y, bk.y);
-            const int o2 = elem(sext_byte<2>(wk), 2, gk.z, bk.z);
-            const int o3 = elem(sext_byte<3>(wk), 3, gk.w, bk.w);
-            out[k] = SAT8 ? (int)pack4_sat_s8(o0, o1, o2, o3) : (int)pack4_s8(o0, o1, o2, o3);
-        }
-        if (live) {
-            int* yr = reinterpret_cast<int*>(y + row * D);
-#pragma unroll
-            for (int k = 0; k < WPL; ++k) __stcs(yr + q + LPR * k, out[k]);
-        }
-    }
-}
-
-// W16 = dim / 16
-template <int W16>
-static int launch_ln_short(const int8_t* x, int8_t* y, int64_t rows, const int32_t* gq, const int32_t* bq,
-                           const uint8_t* ptf_in, const LnDev& c, cudaStream_t st)
-{
-    const int threads = 256;
-    constexpr int LPR = W16 <= 6 ? 2 : 4, WPL = 4 * W16 / LPR;
-    const int64_t want = ((rows + 32 / LPR - 1) / (32 / LPR) + 7) / 8;
-    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * 8);
-    const bool sat8 = c.out.qmin == -128 && c.out.qmax == 127;
-    LnDev cc = c;
-    const long long rz = (long long)c.out.rnd + ((long long)c.out.zp << c.out.shift);
-    const bool zpf = rz > -(1ll << 30) && rz < (1ll << 30);
-    if (zpf) { cc.out.rnd = (int)rz; cc.out.zp = 0; }
-#define IPTQ_LNS_GO(P, S8, ZF) launch_kernel(layernorm_short_rows_kernel<LPR, WPL, P, S8, ZF>, grid, threads, 0, st, x, y, rows, gq, bq, ptf_in, cc)
-    if (c.variant == IPTQ_LN_PTF) { if (sat8) IPTQ_LNS_GO(true, true, false); else IPTQ_LNS_GO(true, false, false); }
-    else if (!sat8)               { IPTQ_LNS_GO(false, false, false); }
-    else if (zpf)                 { IPTQ_LNS_GO(false, true, true); }
-    else                          { IPTQ_LNS_GO(false, true, false); }
-#undef IPTQ_LNS_GO
-    note_launch();
-    return last_launch_status();
-}
-
-template <int NW>
-static int launch_ln(const int8_t* x, int8_t* y, int64_t rows, const int32_t* gq, const int32_t* bq,
-                     const uint8_t* ptf_in, const LnDev& c, cudaStream_t st)
-{
-    constexpr int RW = NW == 1 ? 8 : NW <= 4 ? 4 : NW <= 8 ? 2 : 1;
-    const int threads = 256;
-    const int64_t want = ((rows + RW - 1) / RW + 7) / 8;
-    // Wide rows (640 channels and more: two CTAs per SM): two waves, and the next rows prefetched from two groups per
-    // warp on; with more CTAs a warp has a single group and nothing to prefetch (ViT-Base LayerNorm 16.7 -> 15.3 us).
-    // Narrower rows: four waves and prefetch only for long loops; there the prefetch costs more than it hides
-    // (192 channels, 50 176 rows: 15.2 us against 16.4 - 17.2 us).
-    constexpr int kCtasPerSm = NW >= 5 ? 4 : 8, kPrefetchFrom = NW >= 5 ? 2 : 4;
-    const int grid = (int)std::min<int64_t>(want, (int64_t)sm_count() * kCtasPerSm);
-    const bool sat8 = c.out.qmin == -128 && c.out.qmax == 127;
-    const bool exact = c.dim == 128 * NW;
-    // fold the zero point into the rounding constant when the sum stays clear of 32-bit overflow (|hi32| < 2^30)
-    LnDev cc = c;
-    const long long rz = (long long)c.out.rnd + ((long long)c.out.zp << c.out.shift);
-    const bool zpf = rz > -(1ll << 30) && rz < (1ll << 30);
-    if (zpf) { cc.out.rnd = (int)rz; cc.out.zp = 0; }
-    const bool ptf = c.variant == IPTQ_LN_PTF;
-    const bool pf = (rows + RW - 1) / RW >= (int64_t)kPrefetchFrom * grid * (threads / 32);   // groups per warp
-#define IPTQ_LN_GO(P, S8, EX, ZF)                                                                                        \
-    do {                                                                                                                 \
-        if (pf) launch_kernel(layernorm_rows_kernel<NW, RW, P, S8, EX, ZF, true>, grid, threads, 0, st, x, y, rows, gq, bq, ptf_ptr, cc);  \
-        else    launch_kernel(layernorm_rows_kernel<NW, RW, P, S8, EX, ZF, false>, grid, threads, 0, st, x, y, rows, gq, bq, ptf_ptr, cc); \
-    } while (0)
-    const uint8_t* ptf_ptr = ptf_in;
-    if (ptf)                      { if (sat8) IPTQ_LN_GO(true, true, false, false); else IPTQ_LN_GO(true, false, false, false); }
-    else if (!sat8)               { IPTQ_LN_GO(false, false, false, false); }
-    else if (exact && zpf)        { IPTQ_LN_GO(false, true, true, true); }
-    else if (exact)               { IPTQ_LN_GO(false, true, true, false); }
-    else if (zpf)                 { IPTQ_LN_GO(false, true, false, true); }
-    else                          { IPTQ_LN_GO(false, true, false, false); }
-#undef IPTQ_LN_GO
-    note_launch();
-    return last_launch_status();
-}
-
-// Used by the encoder block as well.
-int layernorm_launch(const int8_t* x, int8_t* y, int64_t rows, int dim, const int32_t* gq, const int32_t* bq,
-                     const uint8_t* ptf, const iptq_ln_consts* consts, cudaStream_t st)
-{
-    if (!consts) return IPTQ_ERR_NULL;
-    if (rows < 0 || dim != consts->dim || dim < 2 || dim > 3072 || (dim & 3)) return IPTQ_ERR_SHAPE;
-    if (rows == 0) return IPTQ_OK;
-    if (!x || !y || !gq || !bq) return IPTQ_ERR_NULL;
-    if (consts->variant < 0 || consts->variant > 2) return IPTQ_ERR_VARIANT;
-    if (consts->variant == IPTQ_LN_PTF && !ptf) return IPTQ_ERR_NULL;
-    if (!aligned16(x) || !aligned16(y) || !aligned16(gq) || !aligned16(bq) ||
-        (ptf && (reinterpret_cast<uintptr_t>(ptf) & 3u)))
-        return IPTQ_ERR_ALIGN;
-    int rc = check_requant(&consts->out);
-    if (rc != IPTQ_OK) return rc;
-    if (rows == 0) return IPTQ_OK;
-    LnDev c;
-    c.variant = consts->variant; c.dim = dim; c.out = to_dev(consts->out);
-    if ((dim & 15) == 0 && dim <= 128 && rows >= 64) {
-        switch (dim / 16) {
-            case 1: return launch_ln_short<1>(x, y, rows, gq, bq, ptf, c, st);
-            case 2: return launch_ln_short<2>(x, y, rows, gq, bq, ptf, c, st);
-            case 3: return launch_ln_short<3>(x, y, rows, gq, bq, ptf, c, st);
-            case 4: return launch_ln_short<4>(x, y, rows, gq, bq, ptf, c, st);
-            case 6: return launch_ln_short<6>(x, y, rows, gq, bq, ptf, c, st);
-            case 8: return launch_ln_short<8>(x, y, rows, gq, bq, ptf, c, st);
-            default: break;                                   // other widths take the general kernel
-        }
-    }
-    const int nw = (dim / 4 + 31) / 32;
-    switch (nw) {
-        case 1: return launch_ln<1>(x, y, rows, gq, bq, ptf, c, st);
-        case 2: return launch_ln<2>(x, y, rows, gq, bq, ptf, c, st);
-        case 3: return launch_ln<3>(x, y, rows, gq, bq, ptf, c, st);
-        case 4: return launch_ln<4>(x, y, rows, gq, bq, ptf, c, st);
-        case 5: case 6: return launch_ln<6>(x, y, rows, gq, bq, ptf, c, st);
-        case 7: case 8: return launch_ln<8>(x, y, rows, gq, bq, ptf, c, st);
-        default:
-            if (nw <= 12) return launch_ln<12>(x, y, rows, gq, bq, ptf, c, st);
-            if (nw <= 16) return launch_ln<16>(x, y, rows, gq, bq, ptf, c, st);
-            return launch_ln<32>(x, y, rows, gq, bq, ptf, c, st);
-    }
-}
-
 }  // namespace iptq
 
 using namespace iptq;
@@ -785,13 +437,6 @@ int iptq_softmax_table(iptq_softmax_consts* consts, uint16_t* table, int32_t cap
     const int rc = last_launch_status();
     if (rc == IPTQ_OK) { consts->table = table; consts->table_n = n; }
     return rc;
-}
-
-int iptq_layernorm(const int8_t* x, int8_t* y, int64_t rows, int dim, const int32_t* gamma_q,
-                   const int32_t* beta_q, const uint8_t* ptf_shift, const iptq_ln_consts* consts,
-                   iptq_stream_t stream)
-{
-    return layernorm_launch(x, y, rows, dim, gamma_q, beta_q, ptf_shift, consts, stream);
 }
 
 }  // extern "C"

@@ -201,6 +201,13 @@ int iptq_layernorm(const int8_t* x, int8_t* y, int64_t rows, int dim, const int3
                    const int32_t* beta_q, const uint8_t* ptf_shift, const iptq_ln_consts* consts,
                    iptq_stream_t stream);
 
+/* The same with row i of the input gathered, without writing it out first: the concatenation over p < parts (1 .. 4) of row
+ * index[i * parts + p] of x, whose rows are dim / parts channels ((dim / parts) % 4 == 0); a negative entry gives zeros
+ * (the 2x2 patch merge of the Swin models).  index: dev int32 [rows, parts]. */
+int iptq_layernorm_gather(const int8_t* x, int8_t* y, int64_t rows, int dim, const int32_t* index, int parts,
+                          const int32_t* gamma_q, const int32_t* beta_q, const uint8_t* ptf_shift,
+                          const iptq_ln_consts* consts, iptq_stream_t stream);
+
 /* ------------------------------------------------------------------ INT8 GEMM carrier
  * Linear ops run in integer arithmetic (Sec. 3.1): acc[m,n] = sum_k x[m,k] w[n,k] + bias[n], which must fit int32
  * (K <= 4096 keeps the sum below 2^26 in magnitude);
@@ -348,10 +355,16 @@ typedef struct {
     int32_t act_bits;              /* width of the QKV / proj / FC2 outputs: 0 or 8 = int8; 6 with 6-bit LayerNorm, Softmax,
                                       attention and GELU constants is the W6A6 setting of the detection results (Sec. 4) */
     const int32_t* attn_bias_t;    /* nullable: attn_bias as laid out by iptq_attention_bias_prepare() (N <= 64) */
+    /* Windows of a token grid (Swin blocks; N <= 64 and B*H >= 2): nullable dev int32 [B*N], the grid row of every window row
+     * (negative: a padding row, zeros in, nothing out); every grid row occurs exactly once.  x and y are then
+     * [grid_rows, D] in grid order: LN1 reads its rows through the index, the attention writes its output rows through it,
+     * and the layers behind it run on grid rows.  Same values as iptq_gather_rows(), the block on window rows,
+     * iptq_gather_rows() back. */
+    const int32_t* window_index; int64_t grid_rows;
 } iptq_block_params;
 
 size_t iptq_encoder_block_workspace_bytes(const iptq_block_params* p /*host*/);
-/* x, y: dev int8 [B*N, D]. */
+/* x, y: dev int8 [B*N, D] ([grid_rows, D] with a window_index). */
 int iptq_encoder_block(const int8_t* x, int8_t* y, const iptq_block_params* p /*host*/, void* ws, size_t ws_bytes,
                        iptq_stream_t stream);
 

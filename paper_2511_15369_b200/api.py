@@ -71,6 +71,7 @@ class BlockParams(C.Structure):
         ("res2_rq", C.c_void_p),
         ("act_bits", C.c_int32),
         ("attn_bias_t", C.c_void_p),
+        ("window_index", C.c_void_p), ("grid_rows", C.c_int64),
     ]
 
 
@@ -186,7 +187,7 @@ def native():
 def exported_symbols():
     """Names declared in include/iptq.h (used by the CPU-side load test)."""
     return ["iptq_requant_prepare", "iptq_channel_requant_prepare", "iptq_softmax_prepare", "iptq_softmax", "iptq_softmax_table",
-            "iptq_gelu_prepare", "iptq_gelu", "iptq_gelu_table", "iptq_gelu_fit", "iptq_gelu_prepare_coeffs", "iptq_layernorm_prepare", "iptq_layernorm",
+            "iptq_gelu_prepare", "iptq_gelu", "iptq_gelu_table", "iptq_gelu_fit", "iptq_gelu_prepare_coeffs", "iptq_layernorm_prepare", "iptq_layernorm", "iptq_layernorm_gather",
             "iptq_unpack_int4", "iptq_linear_workspace_bytes", "iptq_linear_plan", "iptq_linear", "iptq_linear_bits", "iptq_linear_w4_static", "iptq_gather_rows", "iptq_patchify", "iptq_attention_workspace_bytes", "iptq_attention_bias_bytes", "iptq_attention_bias_prepare", "iptq_attention_block",
             "iptq_mlp_workspace_bytes", "iptq_mlp_block", "iptq_encoder_block_workspace_bytes",
             "iptq_encoder_block", "iptq_encoder_block_profiled", "iptq_workspace_init", "iptq_check", "iptq_workspace_set_wait_limit", "iptq_selftest_wait_timeout", "iptq_strerror", "iptq_launch_count",
@@ -412,6 +413,11 @@ def layernorm(x, gamma_q, beta_q, consts: LnConsts, ptf_shift=None, out=None):
     return (_nat or native()).layernorm(x, gamma_q, beta_q, consts, ptf_shift, out)
 
 
+def layernorm_gather(x, index, gamma_q, beta_q, consts: LnConsts, ptf_shift=None, out=None):
+    """``layernorm(gather_rows(x, index), ...)`` without the gathered rows going through memory."""
+    return (_nat or native()).layernorm_gather(x, index, gamma_q, beta_q, consts, ptf_shift, out)
+
+
 def unpack_int4(w_packed):
     """Packed int4 weights [N, K/2] -> int8 [N, K] on the device (what ``w_bits=8`` takes), once at load time."""
     n, k2 = w_packed.shape
@@ -501,7 +507,9 @@ class EncoderBlock:
     (or any object with the same fields) with the library's own ``*_prepare`` functions."""
 
     def __init__(self, spec, table=(SM_BITEXP, GELU_POLY4, LN_SHIFT, LN_SHIFT), device="cuda", gelu_table_on=True,
-                 softmax_table_on=True, unpack_w4_once=False):
+                 softmax_table_on=True, unpack_w4_once=False, window_index=None, grid_rows=0):
+        """window_index: device int32 [B*N], the grid row of every window row (negative: padding); the block then maps
+        [grid_rows, D] to [grid_rows, D] in grid order."""
         sh = spec.shape
         self.shape = sh
         self.keep = []          # host structs and device tensors referenced by raw pointers
@@ -512,6 +520,10 @@ class EncoderBlock:
         p.B, p.N, p.D, p.H, p.dh, p.Dh, p.w_bits = sh.B, sh.N, sh.D, sh.H, sh.dh, sh.Dh, w_bits
         p.table = VariantTable(*table)
         p.act_bits = ab
+        if window_index is not None:
+            assert window_index.numel() == sh.B * sh.N and window_index.dtype == torch.int32
+            self.keep.append(window_index)
+            p.window_index, p.grid_rows = _dp(window_index), int(grid_rows)
         sm_v, gelu_v, ln1_v, ln2_v = table
 
         def dev(a):

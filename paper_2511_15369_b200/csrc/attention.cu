@@ -81,6 +81,7 @@ static int attention_check(const AttnArgs& a)
         (a.tok_stride & 15) || (a.head_stride & 15) || (a.batch_stride & 15))
         return IPTQ_ERR_ALIGN;
     if (a.B * a.H * ((a.N + 127) / 128) > (int64_t)1 << 30) return IPTQ_ERR_SHAPE;
+    if (a.out_index && (a.N > 64 || a.B * a.H < 2)) return IPTQ_ERR_SHAPE;        // the window kernel alone takes it
     return IPTQ_OK;
 }
 
@@ -151,7 +152,7 @@ int attention_launch(const AttnArgs& a, cudaStream_t st)
         while ((int)p.tmem_cols < p.o_col + (a.sm->variant == IPTQ_SM_LOG2 ? 2 : 1) * a.dh) p.tmem_cols <<= 1;
     }
     p.lut_src = (p.lut_n && a.sm->table && a.sm->table_n == p.lut_n) ? a.sm->table : nullptr;
-    p.bias = a.bias; p.mask_id = a.mask_id; p.out = a.out;
+    p.bias = a.bias; p.mask_id = a.mask_id; p.out = a.out; p.out_index = a.out_index;
     p.bias_q = (window && a.bias && a.bias_t) ? reinterpret_cast<const int4*>(a.bias_t) : nullptr;
     p.ex = to_dev_exp(*a.sm);
     p.M = a.sm->M; p.f_shl = a.sm->f_shl; p.p_shr = a.sm->p_shr;

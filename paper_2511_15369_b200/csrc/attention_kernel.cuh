@@ -53,6 +53,7 @@ struct AttnParams {
     const uint16_t* lut_src;   // the same table in device memory (copied), or null (built by each CTA)
     uint32_t tmem_cols;
     const int32_t* bias;   // [H, N, N] or null
+    const int32_t* out_index;   // window kernel: [B * N] output row of every token (negative: none), or null
     const int4* bias_q;    // window kernel: the same bias as [H][ceil(N/4) column quads][64 rows] of 4 columns each, or null
     const uint8_t* mask_id;// [B, N] or null
     int8_t* out;           // [B, N, H*dh]

@@ -30,6 +30,14 @@ template <int DH, int VARIANT> struct WinCfg {
     static_assert(G * GCOLS <= 512, "TMEM");
 };
 
+// A table entry, in a form the compiler cannot issue ahead of the test for a null table.
+__device__ __forceinline__ int load_index(const int32_t* p)
+{
+    int v;
+    asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // FULL: 48 < N <= 64, i.e. every row has its four 16-column chunks (the Swin window of 49 tokens): the chunk loops
 // then carry no run-time conditions.
 template <int DH, int VARIANT, bool HAS_BIAS, bool HAS_MASK, bool PSHR, bool USE_LUT, bool FULL>
@@ -220,6 +228,8 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const int h = bh % p.H, b = bh / p.H;
             const bool valid = exists && row < p.N;
             const bool warp_rows = exists && (quad & 1) * 32 < p.N;     // warp-uniform: any valid row in this warp
+            int64_t dst = valid ? (int64_t)b * p.N + row : -1;          // output row
+            if (p.out_index && valid) dst = load_index(p.out_index + dst);
             // one thread per row: with the row-major bias the 32 lanes of a load hit 32 different sectors and a row
             // takes N loads; the re-laid-out copy gives a thread 4 columns per 16-byte load and a warp 512 contiguous bytes
             const int C4 = (p.N + 3) >> 2;
@@ -357,7 +367,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             if (warp_rows) {
-                int8_t* orow = p.out + ((size_t)b * p.N + row) * HD + h * DH;
+                int8_t* orow = p.out + dst * HD + h * DH;
 #pragma unroll
                 for (int c = 0; c < DH / 16; ++c) {
                     uint32_t r[16];
@@ -377,7 +387,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                         o[j] = requant_nosat((int)r[j], p.orq);
                         if (!sat8) o[j] = max(p.orq.qmin, min(p.orq.qmax, o[j]));
                     }
-                    if (valid) {
+                    if (dst >= 0) {
                         int4 pk;
                         pk.x = (int)pack4_sat_s8(o[0], o[1], o[2], o[3]);
                         pk.y = (int)pack4_sat_s8(o[4], o[5], o[6], o[7]);

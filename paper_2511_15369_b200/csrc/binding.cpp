@@ -22,6 +22,7 @@ struct Api {
     decltype(&iptq_softmax) softmax;
     decltype(&iptq_gelu) gelu;
     decltype(&iptq_layernorm) layernorm;
+    decltype(&iptq_layernorm_gather) layernorm_gather;
     decltype(&iptq_linear_bits) linear_bits;
     decltype(&iptq_gather_rows) gather_rows;
     decltype(&iptq_patchify) patchify;
@@ -191,6 +192,20 @@ PyObject* layernorm(PyObject* const* a, Py_ssize_t)
     check(api.layernorm(static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), x.size(0), (int)x.size(1),
                         dev<int32_t>(a[1]), dev<int32_t>(a[2]), dev<uint8_t>(a[4]), host_struct<iptq_ln_consts>(a[3]), stream()),
           "iptq_layernorm");
+    return out.result();
+}
+
+// layernorm_gather(x, index, gamma_q, beta_q, consts, ptf_shift, out)
+PyObject* layernorm_gather(PyObject* const* a, Py_ssize_t)
+{
+    const at::Tensor& x = device_tensor(a[0]);
+    const at::Tensor& index = device_tensor(a[1]);
+    rank2(x); rank2(index);
+    const int64_t rows = index.size(0), parts = index.size(1), sizes[2] = {rows, parts * x.size(1)};
+    Out out(a[6], sizes, at::kChar, x);
+    check(api.layernorm_gather(static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), rows, (int)sizes[1],
+                               static_cast<const int32_t*>(index.data_ptr()), (int)parts, dev<int32_t>(a[2]), dev<int32_t>(a[3]),
+                               dev<uint8_t>(a[5]), host_struct<iptq_ln_consts>(a[4]), stream()), "iptq_layernorm_gather");
     return out.result();
 }
 
@@ -404,7 +419,7 @@ PyObject* bind(PyObject* const* a, Py_ssize_t)
         fn = reinterpret_cast<std::remove_reference_t<decltype(fn)>>(dlsym(h, name));
         if (!fn) fail(PyExc_ImportError, name);
     };
-    get(api.softmax, "iptq_softmax"); get(api.gelu, "iptq_gelu"); get(api.layernorm, "iptq_layernorm");
+    get(api.softmax, "iptq_softmax"); get(api.gelu, "iptq_gelu"); get(api.layernorm, "iptq_layernorm"); get(api.layernorm_gather, "iptq_layernorm_gather");
     get(api.linear_bits, "iptq_linear_bits"); get(api.gather_rows, "iptq_gather_rows"); get(api.patchify, "iptq_patchify");
     get(api.attention_block, "iptq_attention_block"); get(api.mlp_block, "iptq_mlp_block");
     get(api.encoder_block, "iptq_encoder_block");
@@ -420,7 +435,7 @@ PyObject* bind(PyObject* const* a, Py_ssize_t)
 
 #define IPTQ_ENTRY(f, n) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(&entry<f, n>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
-    IPTQ_ENTRY(bind, 2), IPTQ_ENTRY(softmax, 4), IPTQ_ENTRY(gelu, 3), IPTQ_ENTRY(layernorm, 6), IPTQ_ENTRY(linear, 13),
+    IPTQ_ENTRY(bind, 2), IPTQ_ENTRY(softmax, 4), IPTQ_ENTRY(gelu, 3), IPTQ_ENTRY(layernorm, 6), IPTQ_ENTRY(layernorm_gather, 7), IPTQ_ENTRY(linear, 13),
     IPTQ_ENTRY(gather_rows, 3), IPTQ_ENTRY(patchify, 3), IPTQ_ENTRY(attention_block, 11), IPTQ_ENTRY(mlp_block, 17),
     IPTQ_ENTRY(encoder_block, 5), IPTQ_ENTRY(analyze_softmax, 6), IPTQ_ENTRY(analyze_gelu, 9), IPTQ_ENTRY(analyze_layernorm, 10),
     IPTQ_ENTRY(metric_scores, 4), {nullptr, nullptr, 0, nullptr}};

@@ -16,14 +16,15 @@ static BlockLayout block_layout(const iptq_block_params* p)
 {
     BlockLayout l;
     const size_t T = (size_t)p->B * (size_t)p->N, D = (size_t)p->D, Dh = (size_t)p->Dh;
+    const size_t G = p->window_index ? (size_t)p->grid_rows : T;          // rows behind the attention
     size_t off = kStatusBytes;
     auto take = [&](size_t bytes) { size_t o = off; off += a256(bytes); return o; };
     l.h1 = take(T * D);
     l.qkv = take(T * 3 * D);
-    l.att = take(T * D);
-    l.x1 = take(T * D);
-    l.h2 = take(T * D);
-    l.hid = take(T * Dh);
+    l.att = take(G * D);
+    l.x1 = take(G * D);
+    l.h2 = take(G * D);
+    l.hid = take(G * Dh);
     l.w_qkv = l.w_proj = l.w_fc1 = l.w_fc2 = 0;
     if (p->w_bits == 4) {
         l.w_qkv = take(3 * D * D);
@@ -40,6 +41,8 @@ static int check_block(const iptq_block_params* p)
     if (!p) return IPTQ_ERR_NULL;
     if (p->B < 0 || p->N < 1 || p->D < 16 || p->H < 1 || p->Dh < 16) return IPTQ_ERR_SHAPE;
     if (p->H * p->dh != p->D) return IPTQ_ERR_SHAPE;
+    if (p->window_index && (p->grid_rows < 0 || p->grid_rows > p->B * p->N)) return IPTQ_ERR_SHAPE;
+    if (reinterpret_cast<uintptr_t>(p->window_index) & 3u) return IPTQ_ERR_ALIGN;
     if (p->w_bits != 8 && p->w_bits != 4) return IPTQ_ERR_BITS;
     if (!p->ln1 || !p->ln2 || !p->sm || !p->pv_rq || !p->gelu || !p->res1_rq || !p->res2_rq) return IPTQ_ERR_NULL;
     if (!p->w_qkv || !p->w_proj || !p->w_fc1 || !p->w_fc2) return IPTQ_ERR_NULL;
@@ -80,7 +83,7 @@ static int encoder_block_run(const int8_t* x, int8_t* y, const iptq_block_params
     int8_t* x1 = reinterpret_cast<int8_t*>(base + l.x1);
     int8_t* h2 = reinterpret_cast<int8_t*>(base + l.h2);
     int8_t* hid = reinterpret_cast<int8_t*>(base + l.hid);
-    const int64_t T = p->B * p->N;
+    const int64_t T = p->B * p->N, G = p->window_index ? p->grid_rows : T;
     const int D = p->D, Dh = p->Dh;
     int stage = 0;
     auto mark = [&]() -> int {                     // stage boundary: record the caller's event, if any
@@ -107,7 +110,7 @@ static int encoder_block_run(const int8_t* x, int8_t* y, const iptq_block_params
         if ((rc = unpack_int4_multi_launch(srcs, dsts, ns, 4, stream)) != IPTQ_OK) return rc;   // one launch for the four matrices
     }
 
-    if ((rc = layernorm_launch(LnArgs{x, p->ln1_gamma, p->ln1_beta, p->ln1_ptf, p->ln1}, h1, T, D, stream)) != IPTQ_OK) return rc;
+    if ((rc = layernorm_launch(LnArgs{x, p->ln1_gamma, p->ln1_beta, p->ln1_ptf, p->ln1, p->window_index}, h1, T, D, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
     const int ab = p->act_bits ? p->act_bits : 8;            // width of the QKV / proj / FC2 outputs
     if (ab < 4 || ab > 8) return IPTQ_ERR_BITS;
@@ -116,18 +119,18 @@ static int encoder_block_run(const int8_t* x, int8_t* y, const iptq_block_params
     if ((rc = mark()) != IPTQ_OK) return rc;
     // a row of qkv is [q | k | v]; head h occupies columns h*dh .. of each third
     AttnArgs aa{qkv, qkv + D, qkv + 2 * D, (int64_t)3 * D, (int64_t)p->dh, (int64_t)p->N * 3 * D, att, p->B, p->H, p->N,
-                p->dh, p->attn_bias, p->mask_id, p->sm, p->pv_rq, status, p->attn_bias_t};
+                p->dh, p->attn_bias, p->mask_id, p->sm, p->pv_rq, status, p->attn_bias_t, p->window_index};
     if ((rc = attention_launch(aa, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
-    LinearArgs lp{att, wp, p->b_proj, p->m_proj, p->s_proj, p->proj_zp, x, p->res1_rq, nullptr, x1, T, D, D, status, ab};
+    LinearArgs lp{att, wp, p->b_proj, p->m_proj, p->s_proj, p->proj_zp, x, p->res1_rq, nullptr, x1, G, D, D, status, ab};
     if ((rc = linear_launch(lp, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
-    if ((rc = layernorm_launch(LnArgs{x1, p->ln2_gamma, p->ln2_beta, p->ln2_ptf, p->ln2}, h2, T, D, stream)) != IPTQ_OK) return rc;
+    if ((rc = layernorm_launch(LnArgs{x1, p->ln2_gamma, p->ln2_beta, p->ln2_ptf, p->ln2}, h2, G, D, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
-    LinearArgs l1{h2, w1, p->b_fc1, p->m_fc1, p->s_fc1, 0, nullptr, nullptr, p->gelu, hid, T, Dh, D, status};
+    LinearArgs l1{h2, w1, p->b_fc1, p->m_fc1, p->s_fc1, 0, nullptr, nullptr, p->gelu, hid, G, Dh, D, status};
     if ((rc = linear_launch(l1, stream)) != IPTQ_OK) return rc;
     if ((rc = mark()) != IPTQ_OK) return rc;
-    LinearArgs l2{hid, w2, p->b_fc2, p->m_fc2, p->s_fc2, p->fc2_zp, x1, p->res2_rq, nullptr, y, T, D, Dh, status, ab};
+    LinearArgs l2{hid, w2, p->b_fc2, p->m_fc2, p->s_fc2, p->fc2_zp, x1, p->res2_rq, nullptr, y, G, D, Dh, status, ab};
     if ((rc = linear_launch(l2, stream)) != IPTQ_OK) return rc;
     return mark();
 }

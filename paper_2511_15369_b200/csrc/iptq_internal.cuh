@@ -47,6 +47,7 @@ struct AttnArgs {
     const iptq_softmax_consts* sm; const iptq_requant* out_rq;
     StatusBlock* status;
     const int32_t* bias_t;  // N <= 64: the bias as iptq_attention_bias_prepare() lays it out (16-byte aligned), or null
+    const int32_t* out_index = nullptr;   // N <= 64: [B * N], the row of out that a token's output goes to (negative: none); null: row b N + i
 };
 int attention_launch(const AttnArgs& a, cudaStream_t st);
 

@@ -470,4 +470,12 @@ int iptq_layernorm(const int8_t* x, int8_t* y, int64_t rows, int dim, const int3
     return layernorm_launch(LnArgs{x, gamma_q, beta_q, ptf_shift, consts}, y, rows, dim, stream);
 }
 
+int iptq_layernorm_gather(const int8_t* x, int8_t* y, int64_t rows, int dim, const int32_t* index, int parts,
+                          const int32_t* gamma_q, const int32_t* beta_q, const uint8_t* ptf_shift,
+                          const iptq_ln_consts* consts, iptq_stream_t stream)
+{
+    if (rows > 0 && !index) return IPTQ_ERR_NULL;
+    return layernorm_launch(LnArgs{x, gamma_q, beta_q, ptf_shift, consts, index, parts}, y, rows, dim, stream);
+}
+
 }  // extern "C"

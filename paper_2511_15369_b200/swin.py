@@ -1,6 +1,6 @@
-"""Swin-shaped backbone as a sequence of C-ABI calls: per block a row gather into 7x7 windows (cyclic shift and
-padding folded into the gather table), the integer encoder block on the windows (relative-position bias, attention
-labels), and the gather back; between stages the 2x2 patch merge (gather, integer LayerNorm, INT8 linear).
+"""Swin-shaped backbone as a sequence of C-ABI calls: per block the integer encoder block with the window index of its
+7x7 windows (cyclic shift and padding folded into the table; relative-position bias, attention labels), so that tokens stay in
+grid order between blocks; between stages the 2x2 patch merge (integer LayerNorm of gathered rows, INT8 linear).
 Host logic only: tables and parameters are prepared once, every step of the data path runs in the library."""
 from __future__ import annotations
 
@@ -18,11 +18,8 @@ class SwinBackbone:
         for st in spec.stages:
             C = st["dim"]
             for bspec, shift, fwd, rev in st["blocks"]:
-                blk = api.EncoderBlock(bspec, table, device)
-                n_rows = bspec.shape.T
-                self.layers.append(("block", blk, dev(fwd.reshape(-1, 1)), dev(rev.reshape(-1, 1)),
-                                    torch.empty((n_rows, C), dtype=torch.int8, device=device),
-                                    torch.empty((n_rows, C), dtype=torch.int8, device=device)))
+                self.layers.append(("block", api.EncoderBlock(bspec, table, device, window_index=dev(fwd.reshape(-1)),
+                                                              grid_rows=rev.size)))
             if st["merge"] is not None:
                 m, tab = st["merge"]
                 gq, bq, lc = api.layernorm_prepare(m.gamma, m.beta, m.ln_out_scale, 0)
@@ -33,14 +30,10 @@ class SwinBackbone:
     def __call__(self, x):
         for L in self.layers:
             if L[0] == "block":
-                _, blk, fwd, rev, xw, yw = L
-                api.gather_rows(x, fwd, out=xw)
-                blk(xw, yw)
-                x = api.gather_rows(yw, rev)
+                x = L[1](x)
             else:
                 _, tab, gq, bq, lc, w, mult, shift, ws = L
-                g = api.gather_rows(x, tab)
-                h = api.layernorm(g, gq, bq, lc)
+                h = api.layernorm_gather(x, tab, gq, bq, lc)
                 x = api.linear(h, w, None, mult, shift, ws)
         return x
 
@@ -51,8 +44,10 @@ class SwinBackbone:
     def gemm_ops(self) -> int:
         ops = 0
         for st in self.spec.stages:
-            for bspec, *_ in st["blocks"]:
-                ops += bspec.shape.gemm_ops()
+            for bspec, _, _, rev in st["blocks"]:
+                # LN1, QKV and the attention run on window rows, padding included; the layers behind them on the grid's tokens
+                s = bspec.shape
+                ops += s.gemm_ops() - 2 * (s.T - rev.size) * (s.D * s.D + 2 * s.D * s.Dh)
             if st["merge"] is not None:
                 m, tab = st["merge"]
                 ops += 2 * tab.shape[0] * m.w.shape[0] * m.w.shape[1]

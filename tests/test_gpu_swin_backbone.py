@@ -77,3 +77,37 @@ def test_backbone_matches_the_oracle_composition(api, orc, name, B, stages):
     assert got.shape == want.shape and len(np.unique(want)) > 30
     bad = int((got != want).sum())
     assert bad == 0, "%d of %d elements differ" % (bad, want.size)
+
+
+@pytest.mark.parametrize("N_grid,shift,H,variant", [((9, 13), 3, 3, 0), ((7, 7), 0, 3, 3), ((20, 8), 3, 12, 1)])
+def test_block_on_grid_rows_equals_gather_block_gather(api, N_grid, shift, H, variant):
+    """EncoderBlock with a window index against the three calls it replaces (padding rows, wrapped windows)."""
+    import torch
+    Hh, Ww = N_grid
+    B, D = 2, 32 * H
+    fwd, mask, rev, nW = synth.swin_window_tables(B, Hh, Ww, shift)
+    shape = synth.BlockShape("grid", B * nW, 49, D, H, 32, 4 * D, True)
+    spec = synth.make_block(shape, seed=Hh, mask_id=mask, calib_images=2)
+    x = torch.from_numpy(synth.make_block(synth.BlockShape("x", B, Hh * Ww, D, H, 32, D), seed=1, calib_images=1).x).cuda()
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    table = (variant, 0, 0, 1)
+    plain = api.EncoderBlock(spec, table)
+    want = api.gather_rows(plain(api.gather_rows(x, dev(fwd.reshape(-1, 1)))), dev(rev.reshape(-1, 1)))
+    blk = api.EncoderBlock(spec, table, window_index=dev(fwd.reshape(-1)), grid_rows=rev.size)
+    got = blk(x)
+    blk.ws.check()
+    assert got.shape == want.shape and torch.equal(got, want)
+
+
+@pytest.mark.parametrize("rows,C,parts", [(1, 4, 1), (70, 32, 4), (301, 96, 4), (130, 384, 4), (5000, 48, 3), (90, 64, 1)])
+def test_layernorm_gather_equals_gather_then_layernorm(api, rows, C, parts):
+    import torch
+    g = np.random.default_rng(rows + C)
+    x = torch.from_numpy(g.integers(-128, 128, size=(777, C)).astype(np.int8)).cuda()
+    idx = torch.from_numpy(g.integers(-1, 777, size=(rows, parts)).astype(np.int32)).cuda()
+    dim = C * parts
+    gq, bq, c = api.layernorm_prepare(g.normal(1, 0.1, dim), g.normal(0, 0.1, dim), 8 / 127)
+    gq, bq = torch.from_numpy(gq).cuda(), torch.from_numpy(bq).cuda()
+    got = api.layernorm_gather(x, idx, gq, bq, c)
+    src = x[idx.long().clamp(min=0)] * (idx >= 0).to(torch.int8)[:, :, None]
+    assert torch.equal(got, api.layernorm(src.reshape(rows, dim).contiguous(), gq, bq, c))

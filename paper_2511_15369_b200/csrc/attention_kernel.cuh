@@ -395,8 +395,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                 int hi[4], lo[4];
 #pragma unroll
                                 for (int t = 0; t < 4; ++t) {
-                                    const unsigned code = log2_code(sum, v[i][q4 * 4 + t]);
-                                    const unsigned w16 = code <= 15u ? (0x8000u >> code) : 0u;
+                                    const unsigned w16 = shr_clamp(0x8000u, log2_code_open(sum, v[i][q4 * 4 + t]));    // 0 beyond 15
                                     hi[t] = (int)(w16 >> 8);
                                     lo[t] = (int)(w16 & 0xffu);
                                 }

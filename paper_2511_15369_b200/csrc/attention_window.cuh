@@ -338,8 +338,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                             for (int t = 0; t < 4; ++t) {
                                 if constexpr (VARIANT == IPTQ_SM_LOG2) {
                                     // p = 2^-code as the 16-bit value 2^(15 - code): exactly one byte is non-zero
-                                    const unsigned code = log2_code(sum, v[i][q4 * 4 + t]);
-                                    const unsigned w16 = code <= 15u ? (0x8000u >> code) : 0u;
+                                    const unsigned w16 = shr_clamp(0x8000u, log2_code_open(sum, v[i][q4 * 4 + t]));    // 0 beyond 15
                                     hi[t] = (int)(w16 >> 8);
                                     lo[t] = (int)(w16 & 0xffu);
                                 } else {

@@ -220,15 +220,23 @@ inline int exp_table_entries(const iptq_softmax_consts& sm)
     return n > (1 << 20) ? 0 : (int)n;
 }
 
-// Logarithm candidate: code = round(log2(round(sum / e))) for 0 < e <= sum < 2^31, IPTQ_LOG2_ZERO beyond 15 or for
-// e = 0.  round(sum / e) with halves up is (sum + (e >> 1)) / e: for odd e no multiple of e lies between
-// sum + (e - 1)/2 and sum + e/2.  The rounded logarithm is the position of the leading one, plus the bit below it.
+// Logarithm candidate: code = round(log2(r)), r = round(sum / e) with halves up, for e <= sum; IPTQ_LOG2_ZERO beyond 15 or for
+// e = 0.  r = floor((sum + floor(e / 2)) / e) reaches an integer T exactly where e (2 T - 1) <= 2 sum (an equality is impossible
+// for odd e), and the rounded logarithm (position of the leading one, plus the bit below it) reaches c where r does
+// T = 2 for c = 1 and T = 3 2^(c - 2) from there on.  So code = 0 where 3 e > 2 sum, else 1 + floor(log2(x / y)) with
+// x = 2 sum + e, y = 3 e; that is the difference of their exponents, one less where x's mantissa is the smaller: the difference
+// of the two float patterns, shifted.  y is exact (e < 2^22), and rounding x down moves it past no y 2^k.  The
+// integer division it replaces was the larger part of both kernels that use it: attention over 128 x 12 heads of 197 tokens
+// 304 -> 126 us, the int32 Softmax of its rows 116 -> 60, 4096 x 3 windows 204 -> 75.  The value of the first form may exceed 15.
+__device__ __forceinline__ unsigned log2_code_open(unsigned sum, unsigned e)
+{
+    const unsigned y = 3u * e, x = 2u * sum + e;
+    const int d = __float_as_int(__uint2float_rd(x)) - __float_as_int(__uint2float_rz(y));
+    return y > 2u * sum ? 0u : (unsigned)(1 + (d >> 23));
+}
 __device__ __forceinline__ unsigned log2_code(unsigned sum, unsigned e)
 {
-    if (e == 0) return IPTQ_LOG2_ZERO;
-    const unsigned r = (sum + (e >> 1)) / e;                 // >= 1
-    const int fl = 31 - __clz((int)r);
-    const unsigned code = (unsigned)fl + (fl >= 1 ? ((r >> (fl - 1)) & 1u) : 0u);
+    const unsigned code = log2_code_open(sum, e);
     return code > 15u ? (unsigned)IPTQ_LOG2_ZERO : code;
 }
 

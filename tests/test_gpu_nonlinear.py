@@ -299,3 +299,17 @@ def test_layernorm_degenerate_rows(api, orc, dim, rows):
             _, _, ca = api.layernorm_prepare(gamma, beta, 0.02 * (1 << (8 - out_bits)), zp, out_bits, variant)
             got = api.layernorm(_cu(x), _cu(gq), _cu(bq), ca, None if ptf is None else _cu(ptf)).cpu().numpy()
             assert (got == orc.layernorm(x, gq, bq, co, ptf)).all()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 49, 197, 1024])
+def test_log2_codes_at_every_exponential(api, orc, n):
+    """The code of every exponential a distance can give, against sums from one term (code 0) to the largest: the
+    comparison e (2 T - 1) <= 2 sum that decides a code is met on both sides of its equality."""
+    scale = 1.0 / 700
+    co, ca = orc.softmax_prepare(scale, n, 4, orc.SM_LOG2), api.softmax_prepare(scale, n, 4, api.SM_LOG2)
+    d = np.arange(0, co.dcap + 2, 1 if n <= 197 else 5)
+    s = np.zeros((len(d), n), np.int32)
+    s[:, 0] = -d
+    far = np.random.default_rng(n).integers(0, 2, (len(d), 1)) * np.arange(n) * 3      # half of the rows: a spread of other terms
+    s[:, 1:] -= far[:, 1:].astype(np.int32)
+    assert (api.softmax(_cu(s), ca).cpu().numpy() == orc.softmax(s, co)).all()

@@ -129,9 +129,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (elect_one()) {
                 grid_dep_wait();                                   // q/k/v come from the previous kernel
                 int s = 0; uint32_t ph = 0;
-                for (;;) {
+                // the first item is the CTA's own number (no round trip to the counter ahead of the first load: 8 x 6 heads of 197 tokens
+                // 8.6 -> 7.1 us); the counter hands out those behind the grid, where there are any
+                const bool counted = p.items > (int)gridDim.x;
+                for (int n = 0;; ++n) {
                     if (!mbar_wait_nocall(&kv_empty[s], ph ^ 1u, ctl, p.status, 11)) break;
-                    const int it = atomicAdd(&p.status->work_next, 1);
+                    int it = (int)blockIdx.x;
+                    if (n > 0) it = counted ? (int)gridDim.x + atomicAdd(&p.status->work_next, 1) : p.items;
                     if (it >= p.items) {
                         item_of[s] = -1;
                         mbar_arrive(&kv_full[s]);                  // release: the consumers see the stop mark
@@ -150,7 +154,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 }
                 // the last CTA to finish re-arms the counters for the next launch that uses this workspace
                 __threadfence();
-                if (atomicAdd(&p.status->work_done, 1) == (int)gridDim.x - 1) {
+                if (counted && atomicAdd(&p.status->work_done, 1) == (int)gridDim.x - 1) {
                     p.status->work_next = 0;
                     p.status->work_done = 0;
                     __threadfence();

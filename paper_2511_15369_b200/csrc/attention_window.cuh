@@ -97,9 +97,11 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             grid_dep_wait();                                   // q/k/v come from the previous kernel
             int s = 0; uint32_t ph = 0;
             int stops = 0;                                     // stop marks written so far (every group needs one)
-            for (;;) {
+            const bool counted = p.items > (int)gridDim.x;     // the first item is the CTA's own number, the counter has the others
+            for (int n = 0;; ++n) {
                 if (!mbar_wait(&kv_empty[s], ph ^ 1u, ctl, p.status, 21)) break;
-                const int it = stops ? p.items : atomicAdd(&p.status->work_next, 1);
+                int it = (int)blockIdx.x;
+                if (n > 0) it = counted && !stops ? (int)gridDim.x + atomicAdd(&p.status->work_next, 1) : p.items;
                 if (it >= p.items) {
                     item_of[s] = -1;
                     mbar_arrive(&kv_full[s]);                  // release: the consumers see the stop mark
@@ -122,7 +124,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             }
             // the last CTA to finish re-arms the counters for the next launch that uses this workspace
             __threadfence();
-            if (atomicAdd(&p.status->work_done, 1) == (int)gridDim.x - 1) {
+            if (counted && atomicAdd(&p.status->work_done, 1) == (int)gridDim.x - 1) {
                 p.status->work_next = 0;
                 p.status->work_done = 0;
                 __threadfence();

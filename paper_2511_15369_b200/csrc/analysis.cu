@@ -36,10 +36,11 @@ __device__ __forceinline__ double an_to_double(int v)
 
 // Adds the CTAs' pairs (x2[i], e2[i]), i < n, in an order that depends on the launch alone: lanes by butterfly, warps and
 // CTAs in index order.  The CTA that finishes last does the final sum and leaves the counter at zero.
+template <int THREADS = kAnThreads>
 __device__ __forceinline__ void an_finish(const double (&x2)[kAnMaxCand], const double (&e2)[kAnMaxCand], int n, double* sums,
                                           unsigned* counter, double* partials)
 {
-    __shared__ double sh[2 * kAnMaxCand][kAnThreads / 32];
+    __shared__ double sh[2 * kAnMaxCand][THREADS / 32];
     __shared__ bool last;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
@@ -52,7 +53,8 @@ __device__ __forceinline__ void an_finish(const double (&x2)[kAnMaxCand], const 
     __syncthreads();
     if (threadIdx.x < 2 * n) {
         double t = 0.0;
-        for (int i = 0; i < kAnThreads / 32; ++i) t += sh[threadIdx.x][i];
+#pragma unroll
+        for (int i = 0; i < THREADS / 32; ++i) t += sh[threadIdx.x][i];
         partials[(size_t)blockIdx.x * 2 * kAnMaxCand + threadIdx.x] = t;
         __threadfence();
     }
@@ -61,9 +63,17 @@ __device__ __forceinline__ void an_finish(const double (&x2)[kAnMaxCand], const 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    for (int i = w; i < 2 * n; i += kAnThreads / 32) {
+    for (int i = w; i < 2 * n; i += THREADS / 32) {
         double t = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(partials + (size_t)b * 2 * kAnMaxCand + i);
+        // eight reads in flight: one after the other they were the length of a small layer's whole row loop
+        for (int b0 = lane; b0 < (int)gridDim.x; b0 += 256) {
+            double q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                q[k] = b0 + 32 * k < (int)gridDim.x ? __ldcg(partials + (size_t)(b0 + 32 * k) * 2 * kAnMaxCand + i) : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) t += q[k];
+        }
         t = an_warp_sum(t);
         if (lane == 0) sums[i] = t;
     }
@@ -238,8 +248,14 @@ __device__ __forceinline__ AnGeluTerm an_gelu_term(int x, double in_scale, doubl
 
 // Layers of kAnGeluTableMin elements and more: the terms of all 2^16 codes are tabulated first (2 MB, L2-resident) and an
 // element then costs one 32-byte read and four additions instead of an fp64 erf and three integer functions
-// (2.4 M elements: 54 us evaluated).  Below, the table would cost more than it saves.
-constexpr int64_t kAnGeluTableMin = 1 << 18;
+// (2.4 M elements: 54 us evaluated).  Below, the table would cost more than it saves.  The reads miss L1 line by line; from
+// kAnGeluHistMin on a CTA counts its elements' codes in shared memory and then adds the terms of every code it has seen
+// times its count, so the table is read once per CTA and not once per element.  Per layer, terms read / counted, codes spread
+// over the whole range: 1 M elements 18.3 / 21.9 us, 2.4 M 24.9 / 23.0, 8.4 M 47.7 / 28.4, 33.6 M 143 / 87.
+constexpr int64_t kAnGeluTableMin = 1 << 18, kAnGeluHistMin = 1 << 21;
+constexpr int kAnHistThreads = 1024, kAnHistBytes = 2 * 65536;             // 16-bit counters: 128 KB, one CTA per SM
+constexpr int kAnHistSteps = 15;                                         // 16-byte reads per thread between two emptyings:
+static_assert(4 * kAnHistThreads * kAnHistSteps < 65536, "a counter holds what lies between two emptyings");
 
 __global__ void __launch_bounds__(kAnThreads)
 analyze_gelu_terms_kernel(AnGeluTerm* __restrict__ table, double in_scale, double out_scale, int out_zp,
@@ -280,6 +296,65 @@ analyze_gelu_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, d
     if ((nvec << 2) + first < n) element(__ldg(x + (nvec << 2) + first));
     const double xs[kAnMaxCand] = {x2, x2, x2, x2};
     an_finish(xs, e2, n_cand, sums, counter, partials);
+}
+
+__global__ void __launch_bounds__(kAnHistThreads, 1)
+analyze_gelu_hist_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, double out_scale, int out_zp,
+                         const __grid_constant__ AnGelu a, int n_cand, const AnGeluTerm* table, double* __restrict__ sums,
+                         unsigned* __restrict__ counter, double* __restrict__ partials)
+{
+    extern __shared__ __align__(16) unsigned hist[];                     // word w: the counts of codes 2 w - 32768 and 2 w - 32767
+    const int tid = threadIdx.x;
+    grid_dep_launch();
+    for (int i = tid; i < kAnHistBytes / 16; i += kAnHistThreads) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    grid_dep_wait();
+    double x2 = 0.0, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
+    auto evaluate = [&](int xi) {
+        const AnGeluTerm t = an_gelu_term(xi, in_scale, out_scale, out_zp, a, n_cand);
+        x2 += t.x2; e2[0] += t.e2[0]; e2[1] += t.e2[1]; e2[2] += t.e2[2];
+    };
+    auto element = [&](int xi) {
+        const unsigned c = (unsigned)xi + 32768u;
+        if (c < 65536u) atomicAdd(&hist[c >> 1], c & 1u ? 65536u : 1u);
+        else evaluate(xi);
+    };
+    const int64_t nvec = n >> 2, stride = (int64_t)gridDim.x * kAnHistThreads;
+    const int4* xv = reinterpret_cast<const int4*>(x);
+    for (int64_t base = (int64_t)blockIdx.x * kAnHistThreads; base < nvec; base += kAnHistSteps * stride) {
+        for (int k0 = 0; k0 < kAnHistSteps; k0 += 5) {
+            int4 q[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) {
+                const int64_t i = base + (k0 + k) * stride + tid;
+                if (i < nvec) q[k] = __ldg(xv + i);
+            }
+#pragma unroll
+            for (int k = 0; k < 5; ++k)
+                if (base + (k0 + k) * stride + tid < nvec) { element(q[k].x); element(q[k].y); element(q[k].z); element(q[k].w); }
+        }
+        __syncthreads();
+        const bool more = base + kAnHistSteps * stride < nvec;
+#pragma unroll 4
+        for (int w = tid; w < kAnHistBytes / 4; w += kAnHistThreads) {
+            const unsigned c = hist[w];
+            if (more) hist[w] = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const unsigned m = h ? c >> 16 : c & 0xffffu;
+                if (m) {
+                    double t0, t1, t2, t3;
+                    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(t0), "=d"(t1), "=d"(t2), "=d"(t3) : "l"(table + 2 * w + h));
+                    const double f = an_to_double((int)m);
+                    x2 = fma(f, t0, x2); e2[0] = fma(f, t1, e2[0]); e2[1] = fma(f, t2, e2[1]); e2[2] = fma(f, t3, e2[2]);
+                }
+            }
+        }
+        if (more) __syncthreads();
+    }
+    if (blockIdx.x == 0 && (nvec << 2) + tid < n) evaluate(__ldg(x + (nvec << 2) + tid));
+    const double xs[kAnMaxCand] = {x2, x2, x2, x2};
+    an_finish<kAnHistThreads>(xs, e2, n_cand, sums, counter, partials);
 }
 
 // ------------------------------------------------------------------------------------------------ LayerNorm
@@ -401,27 +476,38 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
         for (int wi = lane; wi < words; wi += 32) {
             const unsigned w = (unsigned)__ldg(xr + wi);
             const unsigned sh = any[1] ? __ldg(reinterpret_cast<const unsigned*>(ptf) + wi) : 0u;
+            // the four channels side by side under each uniform test: a row is one chain of fp64 latencies otherwise
+            int xv[2][4];
+            double2 fp[4];
+            int2 qp[4];
+            double X[2][4];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
-                const int xv[2] = {(int)(int8_t)(w >> (8 * t)), ((int)(int8_t)(w >> (8 * t))) << ((sh >> (8 * t)) & 3)};
-                const double2 fp = gb[4 * wi + t];
-                const int2 qp = gbq[4 * wi + t];
-                double X[2] = {0.0, 0.0};
+                xv[0][t] = (int)(int8_t)(w >> (8 * t));
+                xv[1][t] = xv[0][t] << ((sh >> (8 * t)) & 3);
+                fp[t] = gb[4 * wi + t];
+                qp[t] = gbq[4 * wi + t];
+            }
 #pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    if (any[p]) {
-                        X[p] = fma((an_to_double(xv[p]) - mu[p]) * inv_sd[p], fp.x, fp.y);
-                        x2[p] = fma(X[p], X[p], x2[p]);
+            for (int p = 0; p < 2; ++p) {
+                if (any[p]) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        X[p][t] = fma((an_to_double(xv[p][t]) - mu[p]) * inv_sd[p], fp[t].x, fp[t].y);
+                        x2[p] = fma(X[p][t], X[p][t], x2[p]);
                     }
                 }
+            }
 #pragma unroll
-                for (int i = 0; i < kAnMaxCand; ++i) {
-                    if (i < n_cand && !same[i]) {
-                        const int p = a.variant[i] == IPTQ_LN_PTF ? 1 : 0;
-                        const int u = D * (p ? xv[1] : xv[0]) - (p ? s1[1] : s1[0]);
+            for (int i = 0; i < kAnMaxCand; ++i) {
+                if (i < n_cand && !same[i]) {
+                    const bool p = a.variant[i] == IPTQ_LN_PTF;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const int u = D * (p ? xv[1][t] : xv[0][t]) - (p ? s1[1] : s1[0]);
                         const int nq = f4[i] ? __mulhi(u, f4[i]) : (int)(((long long)u * F[i]) >> 30);
-                        const int o = requant_full(nq * qp.x + qp.y, a.out[i]);
-                        const double d = (p ? X[1] : X[0]) - an_to_double(o - out_zp) * out_scale;
+                        const int o = requant_full(nq * qp[t].x + qp[t].y, a.out[i]);
+                        const double d = (p ? X[1][t] : X[0][t]) - an_to_double(o - out_zp) * out_scale;
                         er[i] = fma(d, d, er[i]);
                     }
                 }
@@ -522,8 +608,21 @@ int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_s
                       n_candidates);
         note_launch();
     }
-    launch_kernel(analyze_gelu_kernel, an_grid((n / 4 + kAnThreads - 1) / kAnThreads, table ? 6 : 4), kAnThreads, 0, stream, x, n, in_scale,
-                  out_scale, out_zp, a, n_candidates, table, sums, counter, partials);
+    if (n >= kAnGeluHistMin) {
+        static bool configured[64];
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return IPTQ_ERR_CUDA;
+        if (!configured[dev]) {
+            if (cudaFuncSetAttribute(analyze_gelu_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnHistBytes) != cudaSuccess)
+                return IPTQ_ERR_CUDA;
+            configured[dev] = true;
+        }
+        launch_kernel(analyze_gelu_hist_kernel, sm_count(), kAnHistThreads, kAnHistBytes, stream, x, n, in_scale, out_scale, out_zp, a,
+                      n_candidates, table, sums, counter, partials);
+    } else {
+        launch_kernel(analyze_gelu_kernel, an_grid((n / 4 + kAnThreads - 1) / kAnThreads, table ? 6 : 4), kAnThreads, 0, stream, x, n,
+                      in_scale, out_scale, out_zp, a, n_candidates, table, sums, counter, partials);
+    }
     note_launch();
     return last_launch_status();
 }

@@ -63,6 +63,23 @@ def test_gelu_candidates(env, orc, n):
         _same(c, metric.error_sums(metric.gelu_float(xq, S), metric.affine_deq(y, So, zp)))
 
 
+@pytest.mark.parametrize("n,constant", [((1 << 21) - 1, False), ((1 << 21) + 3, False), (10_000_003, False), (10_000_000, True)])
+def test_gelu_counted_codes(env, orc, n, constant):
+    """Layers large enough for the kernel that counts codes: every code of the range, a tail that fills no vector, more elements
+    than a counter of one CTA can hold (it is emptied on the way), all of them on one code."""
+    api, assign, metric = env
+    S, So, zp = 2.5e-4, 8.2 / 255, -123
+    xq = np.full(n, -77, np.int32) if constant else np.random.default_rng(n).integers(-32768, 32768, n).astype(np.int32)
+    an = assign.Analyzer()
+    layer = an.gelu_layer("x", _cu(xq), S, 16, So, zp)
+    an.finish()
+    codes, counts = np.unique(xq, return_counts=True)
+    X = metric.gelu_float(codes, S)
+    for c in layer.candidates:
+        d = X - metric.affine_deq(orc.gelu(codes, orc.gelu_prepare(S, 16, So, zp, 8, c.variant)), So, zp)
+        _same(c, (float((counts * X * X).sum()), float((counts * d * d).sum())))
+
+
 @pytest.mark.parametrize("rows,dim", [(1, 4), (9, 100), (33, 128), (197, 192), (50, 768), (7, 3072)])
 def test_layernorm_candidates(env, orc, rows, dim):
     api, assign, metric = env

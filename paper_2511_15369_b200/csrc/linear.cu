@@ -224,19 +224,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     const int stages = p.stages;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
 
-    if (warp == 0) {
-        // the barriers lie one behind the other: full, empty, acc_full, acc_empty, res_bar; a lane initialises one or two
-        const int n_acc = 2 * MAX_STAGES + 2;                  // first acc_empty
-        for (int i = lane; i < n_acc + 2 + (EPI == EPI_RESIDUAL ? 2 * EPI_WARPS : 0); i += 32)
-            mbar_init(&full_bar[i], i >= n_acc && i < n_acc + 2 ? (PAIR ? 2 * EPI_WARPS : EPI_WARPS) : 1);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < MAX_STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], PAIR ? 2 * EPI_WARPS : EPI_WARPS); }
+        for (int w = 0; w < 2 * EPI_WARPS; ++w) mbar_init(&res_bar[w], 1);
+        ctl->abort = 0;
         fence_barrier_init();
-        if (lane == 0) {
-            ctl->abort = 0;
-            prefetch_tensormap(&map_w);
-            prefetch_tensormap(&map_x);
-            prefetch_tensormap(&map_y);
-            if (EPI == EPI_RESIDUAL) prefetch_tensormap(&map_res);
-        }
+        prefetch_tensormap(&map_w);
+        prefetch_tensormap(&map_x);
+        prefetch_tensormap(&map_y);
+        if (EPI == EPI_RESIDUAL) prefetch_tensormap(&map_res);
     }
     if (warp == 1) {
         if (PAIR) { tmem_alloc_pair(tmem_slot, TMEM_COLS); tmem_relinquish_pair(); }
@@ -456,8 +453,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             if (EPI == EPI_RESIDUAL && !two && nhave) request_residual(ntt, nct, 0);
             have = nhave; tt = ntt; ct = nct; cm = ncm; cs = ncs; cb = ncb;
         }
-        // the stores have read shared memory before it goes away; that they have written is part of the launch's completion
-        if (lane == 0) bulk_wait_read_all();
+        if (lane == 0) bulk_wait_all();                       // stores complete before shared memory goes away
     }
 
     // ------------------------------------------------------------ teardown (also reached after an abort)

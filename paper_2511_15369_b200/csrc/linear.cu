@@ -679,13 +679,6 @@ static int gemm_plan(GemmParams& p, int64_t M, bool residual, bool table, int sm
     if (small) {
         const int64_t tiles64 = (int64_t)p.n_ct * ((M + 63) / 64);
         best_tn = tiles64 <= sms ? 64 : 128;
-        // Where even the full tiles of 128 tokens take a second round but 192-token tiles fit one, these win (1182 tokens, 768 x 2304
-        // 6.5 -> 5.6 us; 2364, 384 x 1152 5.3 -> 4.8; 2048, 384 x 1536 6.6 -> 6.0); where only ragged ones are left over they lose
-        // (788 tokens, 768 x 3072: 6.4 at 128, 7.1 at 192).
-        GemmParams q = p;
-        int sb;
-        if (best_tn == 128 && p.n_ct * (M / 128) > sms && p.n_ct * ((M + 191) / 192) <= sms &&
-            gemm_layout(q, 192, false, residual, table, kblocks, 1, &sb) >= std::min(3, kblocks + 1)) best_tn = 192;
     } else if (pair) best_tn = 256;
     else for (int TN : {256, 192, 128, 64}) {
         if (narrow && TN > 128) continue;

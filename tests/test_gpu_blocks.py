@@ -71,13 +71,6 @@ def test_linear_parity(api, orc, M, N, K):
     assert (got == want).all(), _mismatch(got, want)
 
 
-@pytest.mark.parametrize("M,N,K", [(2364, 1152, 384), (1153, 2304, 768), (2305, 1104, 112)])
-def test_linear_one_round_of_192_token_tiles(api, orc, M, N, K):
-    """Shapes whose 128-token tiles would take a second round: a ragged last tile of 60 tokens, of one, of one with ragged channels."""
-    assert api.linear_plan(M, N, K, sm_count=148).tile_tokens == 192
-    test_linear_parity(api, orc, M, N, K)
-
-
 @pytest.mark.parametrize("M,N,K", [(300, 160, 96), (2600, 384, 1536)])
 def test_linear_large_shifts_and_biases(api, orc, M, N, K):
     """Channel groups whose shifts are all small, all large and mixed (the epilogue treats the zero point differently

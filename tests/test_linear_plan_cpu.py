@@ -75,10 +75,3 @@ def test_shapes_the_layer_rejects_are_rejected_by_the_plan():
     for M, N, K in [(0, 128, 128), (128, 8, 128), (128, 128, 8), (128, 130, 128), (128, 128, 4112), (128, 128, 100)]:
         with pytest.raises(api.IptqError):
             plan(M, N, K)
-
-
-def test_one_round_of_192_token_tiles_instead_of_two_of_128():
-    assert plan(1182, 2304, 768).tile_tokens == 192 and plan(1182, 2304, 768).grid == 18 * 7
-    assert plan(2364, 1152, 384).tile_tokens == 192 and plan(2048, 1536, 384, gelu_table=True).tile_tokens == 192
-    assert plan(788, 3072, 768, gelu_table=True).tile_tokens == 128      # 24 x 6 full tiles fit a round, the ragged 24 are short
-    assert plan(3152, 1152, 384).tile_tokens == 128                      # 9 x 17 tiles of 192 tokens do not fit one

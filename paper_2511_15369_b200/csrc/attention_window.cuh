@@ -396,6 +396,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
                         pk.w = (int)pack4_sat_s8(o[12], o[13], o[14], o[15]);
                         *reinterpret_cast<int4*>(orow + c * 16) = pk;
                     }
+                    __syncwarp();                              // rows without an output leave gaps in the warp: joined before the next TMEM load
                 }
             }
             tc_fence_before_sync();

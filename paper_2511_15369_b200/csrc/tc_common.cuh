@@ -194,8 +194,8 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 32 lanes x 16 consecutive 32-bit columns: thread t of the warp gets lane (quadrant*32 + t).
-// .aligned: every lane must be there, so a __syncwarp() stands between the last mbarrier wait (after which some lanes may
-// still be polling) and the first load.
+// .aligned: every lane must be there, so a __syncwarp() stands between the load and whatever may have split the warp before
+// it: an mbarrier wait (after which some lanes may still be polling) or a branch that only some lanes take.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(

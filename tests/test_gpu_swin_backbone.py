@@ -99,6 +99,25 @@ def test_block_on_grid_rows_equals_gather_block_gather(api, N_grid, shift, H, va
     assert got.shape == want.shape and torch.equal(got, want)
 
 
+@pytest.mark.parametrize("variant", [0, 3])
+@pytest.mark.parametrize("grid,shift,H", [((10, 12), 3, 3), ((8, 8), 0, 2)])
+def test_block_on_grid_rows_with_wide_heads(api, grid, shift, H, variant):
+    """As above with heads of 64: an output row goes out in four pieces, and most windows have rows without an output."""
+    import torch
+    B, D = 2, 64 * H
+    fwd, mask, rev, nW = synth.swin_window_tables(B, *grid, shift)
+    assert (fwd < 0).any()
+    spec = synth.make_block(synth.BlockShape("grid", B * nW, 49, D, H, 64, 4 * D, True), seed=H, mask_id=mask, calib_images=2)
+    x = torch.from_numpy(np.random.default_rng(H).integers(-128, 128, size=(rev.size, D)).astype(np.int8)).cuda()
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    table = (variant, 0, 0, 0)
+    want = api.gather_rows(api.EncoderBlock(spec, table)(api.gather_rows(x, dev(fwd.reshape(-1, 1)))), dev(rev.reshape(-1, 1)))
+    blk = api.EncoderBlock(spec, table, window_index=dev(fwd.reshape(-1)), grid_rows=rev.size)
+    got = blk(x)
+    blk.ws.check()
+    assert torch.equal(got, want)
+
+
 @pytest.mark.parametrize("rows,C,parts", [(1, 4, 1), (70, 32, 4), (301, 96, 4), (130, 384, 4), (5000, 48, 3), (90, 64, 1)])
 def test_layernorm_gather_equals_gather_then_layernorm(api, rows, C, parts):
     import torch

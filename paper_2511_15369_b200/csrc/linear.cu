@@ -142,13 +142,16 @@ __device__ __forceinline__ int tile_tokens(const GemmParams& p, int tt)
 // the warp's staging block.  Straight-line code: tile width, output range and the place of the zero point are template
 // parameters, because the tests and reconvergence points they would otherwise put into every chunk of 16 tokens were
 // a third of the epilogue's instructions, and the epilogue is bound by the instructions it issues.
-// acc[0] holds chunk 0 (its load is in flight); hand_back() is called once the last load has completed.
+// No load is in flight across the choice between the copies of this function; hand_back() is called once the last one
+// has completed.
 // ZP_AFTER: the output zero point is added behind the shift instead of being part of crnd.
 template <int EPI, int GELU_VARIANT, int NCH, bool SAT8, bool ZP_AFTER, typename HandBack>
-__device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, uint32_t (&acc)[2][16], int cm, int cs,
-                                              int cb, int crnd, uint32_t res_lane, uint32_t tab_mid, uint32_t out_word,
+__device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, int cm, int cs, int cb,
+                                              int crnd, uint32_t res_lane, uint32_t tab_mid, uint32_t out_word,
                                               unsigned sel1, unsigned sel2, HandBack&& hand_back)
 {
+    uint32_t acc[2][16];
+    tmem_ld16(tacc, acc[0]);
 #pragma unroll
     for (int ch = 0; ch < NCH; ++ch) {
         tmem_wait_ld();                                        // chunk ch is in registers
@@ -430,15 +433,13 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 // A wait can split the warp (its lanes try one after the other, and the barrier may complete in between), and
                 // the TMEM loads are .aligned: without this the compiler need not have joined the lanes again.
                 __syncwarp();
-                uint32_t acc[2][16];
-                tmem_ld16(tacc, acc[0]);
                 const uint32_t tab = EPI == EPI_RESIDUAL ? rlut_mid : tab_mid;
                 if (!fold)
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, true>(p, tacc, acc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
+                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, true>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
                 else if (EPI == EPI_GELU_TAB || sat8)
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, true, false>(p, tacc, acc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
+                    epilogue_tile<EPI, GELU_VARIANT, NCH, true, false>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
                 else
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, false>(p, tacc, acc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
+                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, false>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
                 fence_proxy_async_smem();                     // this lane's shared-memory stores -> visible to the TMA engine
                 __syncwarp();
                 if (lane == 0) {

@@ -248,8 +248,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 
         // requantises and stores this thread's share of the output tile of item (b, h, mt), count index k
         auto epilogue = [&](int k, int b, int h, int mt) -> bool {
-            if (!mbar_wait_nocall(o_full, (uint32_t)k & 1u, ctl, p.status, 16)) return false;
-            __syncwarp();                                      // the wait may have split the warp
+            if (!mbar_wait_warp<false>(o_full, (uint32_t)k & 1u, ctl, p.status, 16)) return false;
             tc_fence_after_sync();
             const int row = mt * 128 + rloc;
             constexpr int OPARTS = DH / 16;                    // threads of a row that hold 16 output columns each
@@ -292,7 +291,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         for (;; ++k) {
             // the four warps of a quadrant meet at two named barriers per item: a warp that gives up before them
             // arrives without waiting, so that a bounded wait running out can never strand the others
-            if (!mbar_wait_nocall(&kv_full[s], ph, ctl, p.status, 17)) {   // acquire: the item number is visible
+            if (!mbar_wait_warp<false>(&kv_full[s], ph, ctl, p.status, 17)) {   // acquire: the item number is visible
                 named_barrier_arrive(1 + quad, 128); named_barrier_arrive(1 + quad, 128);
                 ok = false;
                 break;
@@ -311,12 +310,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const unsigned my_id = HAS_MASK ? mrow[valid ? row : 0] : 0u;
             const uint32_t p_row = p_row0 + (uint32_t)((k & 1) * p.p_bytes);
 
-            if (!mbar_wait_nocall(s_full, (uint32_t)k & 1u, ctl, p.status, 15)) {
+            if (!mbar_wait_warp<false>(s_full, (uint32_t)k & 1u, ctl, p.status, 15)) {
                 named_barrier_arrive(1 + quad, 128); named_barrier_arrive(1 + quad, 128);
                 ok = false;
                 break;
             }
-            __syncwarp();                                      // the wait may have split the warp
             tc_fence_after_sync();
             // ---- this thread's quarter of the score row, TMEM -> registers, in one batch
             uint32_t v[4][16];

@@ -221,7 +221,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 
         for (int k = g, n = 0;; k += G, ++n) {
             const int sk = k % ST;
-            if (!mbar_wait(&kv_full[sk], (uint32_t)(k / ST) & 1u, ctl, p.status, 27)) break;   // acquire: the item number is visible
+            if (!mbar_wait_warp(&kv_full[sk], (uint32_t)(k / ST) & 1u, ctl, p.status, 27)) break;   // acquire: the item number is visible
             const int it = item_of[sk];
             if (it < 0) break;
             int bh = 2 * it + win;
@@ -250,8 +250,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             const unsigned id_lo = HAS_MASK && lane < p.N ? mrow[lane] : 0x100u;
             const unsigned id_hi = HAS_MASK && lane + 32 < p.N ? mrow[lane + 32] : 0x100u;
 
-            if (!mbar_wait(&s_full[g], (uint32_t)n & 1u, ctl, p.status, 25)) break;
-            __syncwarp();                                      // the wait may have split the warp
+            if (!mbar_wait_warp(&s_full[g], (uint32_t)n & 1u, ctl, p.status, 25)) break;
             tc_fence_after_sync();
             uint32_t v[4][16];
 #pragma unroll
@@ -364,8 +363,7 @@ window_attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(&p_ready[g]);
             // ---- output of this item: the other groups' items fill the time the P V product takes
-            if (!mbar_wait(&o_full[g], (uint32_t)n & 1u, ctl, p.status, 26)) break;
-            __syncwarp();                                      // the wait may have split the warp
+            if (!mbar_wait_warp(&o_full[g], (uint32_t)n & 1u, ctl, p.status, 26)) break;
             tc_fence_after_sync();
             if (warp_rows) {
                 int8_t* orow = p.out + dst * HD + h * DH;

@@ -412,7 +412,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             // epilogue has it in the table of residual terms, the GELU epilogues have none.
             const bool fold = EPI != EPI_REQUANT || __all_sync(0xffffffffu, cs <= 20);
             const int crnd = (1 << (cs - 1)) + (EPI == EPI_REQUANT && fold ? p.out_zp << cs : 0);
-            if (!mbar_wait(&acc_full[ab], abph, ctl, p.status, 4)) break;
+            if (!mbar_wait_warp(&acc_full[ab], abph, ctl, p.status, 4)) break;
             tc_fence_after_sync();
             const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * ACC_COLS + part * tpp);
             auto hand_back = [&] {                             // the MMA warp may refill this accumulator
@@ -427,12 +427,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
                 if (lane == 0) { if (two) bulk_wait_read_but_one(); else bulk_wait_read_all(); }
                 __syncwarp();
                 if (EPI == EPI_RESIDUAL) {
-                    if (!mbar_wait(&res_bar[2 * ew + sb], (res_ph >> sb) & 1u, ctl, p.status, 5)) break;
+                    if (!mbar_wait_warp(&res_bar[2 * ew + sb], (res_ph >> sb) & 1u, ctl, p.status, 5)) break;
                     res_ph ^= 1u << sb;
                 }
-                // A wait can split the warp (its lanes try one after the other, and the barrier may complete in between), and
-                // the TMEM loads are .aligned: without this the compiler need not have joined the lanes again.
-                __syncwarp();
                 const uint32_t tab = EPI == EPI_RESIDUAL ? rlut_mid : tab_mid;
                 if (!fold)
                     epilogue_tile<EPI, GELU_VARIANT, NCH, false, true>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);

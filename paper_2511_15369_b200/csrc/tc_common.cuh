@@ -118,15 +118,19 @@ __device__ __forceinline__ bool mbar_wait_nocall(uint64_t* bar, uint32_t parity,
     return mbar_wait_poll(bar, parity, ctl, status, where);
 }
 
-// The same wait for a whole (converged) warp: one lane polls, the others learn the outcome from a shuffle, which
-// also orders the warp's later reads behind the wait.  Several hundred threads polling one barrier word take
-// turns on it, about two clocks each: a wait that is already satisfied then costs a thousand clocks.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, CtaControl* ctl, StatusBlock* status,
-                                               int where)
+// The same wait for a whole warp: one lane polls, the others learn the outcome from a shuffle and come behind its acquire
+// through the barrier.  With every lane polling, a barrier that completes between the lanes' tries splits the warp, and
+// what follows these waits (TMEM loads, register reallocation, named barriers) is .aligned; the warp is whole when this
+// returns, and all its lanes go the same way.
+template <bool CALL = true>
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, CtaControl* ctl, StatusBlock* status, int where)
 {
     int ok = 1;
-    if ((threadIdx.x & 31u) == 0) ok = mbar_wait(bar, parity, ctl, status, where) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    if ((threadIdx.x & 31u) == 0)
+        ok = CALL ? mbar_wait(bar, parity, ctl, status, where) : mbar_wait_nocall(bar, parity, ctl, status, where);
+    ok = __shfl_sync(0xffffffffu, ok, 0);
+    __syncwarp();
+    return ok != 0;
 }
 
 // ---------------------------------------------------------------- TMA tile copies, one CTA per copy

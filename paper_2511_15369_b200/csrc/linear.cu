@@ -594,7 +594,9 @@ static int launch_gemm(const CUtensorMap& mw, const CUtensorMap& mx, const CUten
     switch (p.TN) {
         case 64: return launch_gemm_as<EPI, GV, false, 1>(mw, mx, my, mr, p, grid, smem_bytes, st);
         case 128: return launch_gemm_as<EPI, GV, false, 2>(mw, mx, my, mr, p, grid, smem_bytes, st);
-        case 192: return launch_gemm_as<EPI, GV, false, 3>(mw, mx, my, mr, p, grid, smem_bytes, st);
+        case 192:
+            if constexpr (EPI == EPI_GELU_TAB) return launch_gemm_as<EPI, GV, false, 3>(mw, mx, my, mr, p, grid, smem_bytes, st);
+            else return IPTQ_ERR_SHAPE;                       // never planned
         default: return launch_gemm_as<EPI, GV, false, 4>(mw, mx, my, mr, p, grid, smem_bytes, st);
     }
 }
@@ -683,6 +685,7 @@ static int gemm_plan(GemmParams& p, int64_t M, bool residual, bool table, int sm
         GemmParams q = p;
         int sb;
         if (TN > 64 && M <= TN - 64) continue;                // a narrower tile covers all tokens
+        if (TN == 192 && !table) continue;                    // that width stands in for 256 beside the GELU table, and is built for it alone
         if (gemm_layout(q, TN, false, residual, table, kblocks, 1, &sb) < std::min(3, kblocks + 1)) continue;
         best_tn = TN;
         break;

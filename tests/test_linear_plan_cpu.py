@@ -51,6 +51,14 @@ def test_small_batches_take_narrow_tiles():
     assert plan(12608, 384, 384, residual=True).tile_tokens == 256
 
 
+def test_192_token_tiles_are_planned_beside_the_gelu_table_alone():
+    # 129 to 192 tokens and more channel tiles than SMs: the one place where other epilogues would get that width
+    for M, N, sms in [(160, 19200, 148), (129, 19200, 148), (192, 2048, 8), (150, 384, 1)]:
+        for residual in (False, True):
+            assert plan(M, N, 384, residual=residual, sm_count=sms).tile_tokens == 128
+    assert plan(12608, 1536, 384, gelu_table=True).tile_tokens == 192
+
+
 def test_the_configurations_of_the_benchmark():
     # short reductions have room for two staging buffers per epilogue warp, the long ones of ViT-Base keep their ring
     assert plan(200704, 96, 96, residual=True).staging_buffers == 2 and plan(200704, 288, 96).staging_buffers == 2

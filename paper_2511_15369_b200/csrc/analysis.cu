@@ -17,9 +17,10 @@ namespace iptq {
 constexpr unsigned kAllLanes = 0xffffffffu;
 constexpr int kAnThreads = 256;
 constexpr int kAnMaxCand = IPTQ_ANALYZE_MAX_CANDIDATES;
-// scratch: the counter (256 bytes), the CTAs' pairs, the GELU terms
+// scratch: the counter (256 bytes), the CTAs' pairs, the GELU terms.  The scratch is 16-byte aligned and a term is read with
+// one 32-byte load, so the terms start at the 32-byte boundary at or below kAnPartialBytes; the pairs end 32 bytes ahead of it.
 constexpr int kAnPartialBytes = 131072;
-constexpr int kAnMaxBlocks = (kAnPartialBytes - 256) / (16 * kAnMaxCand);
+constexpr int kAnMaxBlocks = (kAnPartialBytes - 256 - 32) / (16 * kAnMaxCand);
 
 __device__ __forceinline__ double an_warp_sum(double v)
 {
@@ -609,7 +610,7 @@ int iptq_analyze_gelu(const int32_t* x, int64_t n, double in_scale, double out_s
     double* partials = reinterpret_cast<double*>(static_cast<uint8_t*>(work) + 256);
     AnGeluTerm* table = nullptr;
     if (n >= kAnGeluTableMin) {
-        table = reinterpret_cast<AnGeluTerm*>(static_cast<uint8_t*>(work) + kAnPartialBytes);
+        table = reinterpret_cast<AnGeluTerm*>((reinterpret_cast<uintptr_t>(work) + kAnPartialBytes) & ~uintptr_t(31));
         launch_kernel(analyze_gelu_terms_kernel, 65536 / kAnThreads, kAnThreads, 0, stream, table, in_scale, out_scale, out_zp, a,
                       n_candidates);
         note_launch();

@@ -112,3 +112,27 @@ def test_sums_are_the_same_bits_twice_and_the_capacity_is_kept(env):
     a, b = an.layers
     an.finish()
     assert [(c.sum_x2, c.sum_err2) for c in a.candidates] == [(c.sum_x2, c.sum_err2) for c in b.candidates]
+
+
+@pytest.mark.parametrize("n", [1 << 18, (1 << 21) + 3])
+def test_scratch_at_every_alignment_the_header_admits(env, n):
+    """Scratch on a 16-byte boundary that is no 32-byte boundary: the terms of the codes are read 32 bytes at a time."""
+    import ctypes as C
+
+    import torch
+    api, assign, metric = env
+    x = _cu(np.random.default_rng(n).integers(-32768, 32768, n).astype(np.int32))
+    consts = (api.GeluConsts * 2)(api.gelu_prepare(2.5e-4, 16, 8.2 / 255, -123), api.gelu_prepare(2.5e-4, 16, 8.2 / 255, -123, 8, 1))
+    got = []
+    for off in (0, 16):
+        buf = torch.zeros(api.ANALYZE_WORK_BYTES + 64, dtype=torch.uint8, device="cuda")
+        guard = off + api.ANALYZE_WORK_BYTES
+        buf[:off] = 0xAB
+        buf[guard:] = 0xAB
+        sums = torch.zeros(4, dtype=torch.float64, device="cuda")
+        assert buf.data_ptr() % 32 == 0
+        assert api.lib().iptq_analyze_gelu(x.data_ptr(), n, 2.5e-4, 8.2 / 255, -123, C.cast(consts, C.c_void_p), 2, sums.data_ptr(),
+                                           buf.data_ptr() + off, torch.cuda.current_stream().cuda_stream) == api.OK
+        got.append(sums.cpu().numpy())
+        assert (buf[:off] == 0xAB).all() and (buf[guard:] == 0xAB).all()
+    assert (got[0] == got[1]).all() and (got[0] > 0).all()

@@ -236,6 +236,15 @@ struct AnGeluTerm {
 };
 static_assert(sizeof(AnGeluTerm) == 32, "one 32-byte sector per code");
 
+// A term of the table that the launch before has written: volatile and a memory operation to the compiler, so that it stays behind
+// the dependency wait and behind the test for a table and the code's range.
+__device__ __forceinline__ AnGeluTerm an_load_term(const AnGeluTerm* p)
+{
+    AnGeluTerm t;
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(t.x2), "=d"(t.e2[0]), "=d"(t.e2[1]), "=d"(t.e2[2]) : "l"(p) : "memory");
+    return t;
+}
+
 __device__ __forceinline__ AnGeluTerm an_gelu_term(int x, double in_scale, double out_scale, int out_zp, const AnGelu& a, int n_cand)
 {
     const double v = an_to_double(x) * in_scale;
@@ -284,15 +293,10 @@ analyze_gelu_kernel(const int32_t* __restrict__ x, int64_t n, double in_scale, d
     grid_dep_wait();
     double x2 = 0.0, e2[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
     auto element = [&](int xi) {
-        if (table && xi >= -32768 && xi < 32768) {
-            // one 256-bit load per element, cached in L1: calibration activations fall on a few thousand codes
-            double t0, t1, t2, t3;
-            asm("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(t0), "=d"(t1), "=d"(t2), "=d"(t3) : "l"(table + 32768 + xi));
-            x2 += t0; e2[0] += t1; e2[1] += t2; e2[2] += t3;
-        } else {
-            const AnGeluTerm t = an_gelu_term(xi, in_scale, out_scale, out_zp, a, n_cand);
-            x2 += t.x2; e2[0] += t.e2[0]; e2[1] += t.e2[1]; e2[2] += t.e2[2];
-        }
+        // one 256-bit load per element, cached in L1: calibration activations fall on a few thousand codes
+        const AnGeluTerm t = table && xi >= -32768 && xi < 32768 ? an_load_term(table + 32768 + xi)
+                                                                : an_gelu_term(xi, in_scale, out_scale, out_zp, a, n_cand);
+        x2 += t.x2; e2[0] += t.e2[0]; e2[1] += t.e2[1]; e2[2] += t.e2[2];
     };
     const int64_t nvec = n >> 2, stride = (int64_t)gridDim.x * kAnThreads, first = (int64_t)blockIdx.x * kAnThreads + threadIdx.x;
     const int4* xv = reinterpret_cast<const int4*>(x);
@@ -350,10 +354,9 @@ analyze_gelu_hist_kernel(const int32_t* __restrict__ x, int64_t n, double in_sca
             for (int h = 0; h < 2; ++h) {
                 const unsigned m = h ? c >> 16 : c & 0xffffu;
                 if (m) {
-                    double t0, t1, t2, t3;
-                    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(t0), "=d"(t1), "=d"(t2), "=d"(t3) : "l"(table + 2 * w + h));
+                    const AnGeluTerm t = an_load_term(table + 2 * w + h);
                     const double f = an_to_double((int)m);
-                    x2 = fma(f, t0, x2); e2[0] = fma(f, t1, e2[0]); e2[1] = fma(f, t2, e2[1]); e2[2] = fma(f, t3, e2[2]);
+                    x2 = fma(f, t.x2, x2); e2[0] = fma(f, t.e2[0], e2[0]); e2[1] = fma(f, t.e2[1], e2[1]); e2[2] = fma(f, t.e2[2], e2[2]);
                 }
             }
         }

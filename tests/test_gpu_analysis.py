@@ -136,3 +136,19 @@ def test_scratch_at_every_alignment_the_header_admits(env, n):
         got.append(sums.cpu().numpy())
         assert (buf[:off] == 0xAB).all() and (buf[guard:] == 0xAB).all()
     assert (got[0] == got[1]).all() and (got[0] > 0).all()
+
+
+@pytest.mark.parametrize("n", [9, 4097, (1 << 18) + 2, (1 << 21) + 1])
+def test_codes_beyond_the_table(env, orc, n):
+    """Inputs wider than 16 bits among the others, in vectors and in the tail, with and without a table of terms."""
+    api, assign, metric = env
+    S, So, zp = 2.5e-4, 8.2 / 255, -123
+    x = np.random.default_rng(n).integers(-32768, 32768, n).astype(np.int32)
+    x[::3] = np.tile([-32769, 32768, 1 << 20, -(1 << 22)], n)[:x[::3].size]
+    x[-1] = 70000
+    an = assign.Analyzer()
+    layer = an.gelu_layer("x", _cu(x), S, 16, So, zp)
+    an.finish()
+    X = metric.gelu_float(x, S)
+    for c in layer.candidates:
+        _same(c, metric.error_sums(X, metric.affine_deq(orc.gelu(x, orc.gelu_prepare(S, 16, So, zp, 8, c.variant)), So, zp)))

@@ -400,7 +400,7 @@ constexpr int kAnLnBytesPerChannel = 24;                                 // shar
 // second time from L1); the parameters wait in shared memory.  Bound by latency at calibration sizes (a few rows per warp).
 template <int MAXD>
 __global__ void __launch_bounds__(kAnThreads)
-analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, const __grid_constant__ AnLnParams<MAXD> prm,
+analyze_layernorm_kernel(const int8_t* x, int64_t rows, int D, const __grid_constant__ AnLnParams<MAXD> prm,
                          const uint8_t* __restrict__ ptf, double out_scale, int out_zp, const __grid_constant__ AnLayerNorm a,
                          int n_cand, double* __restrict__ sums, unsigned* __restrict__ counter, double* __restrict__ partials)
 {
@@ -434,7 +434,7 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
         int s1[2] = {0, 0};
         unsigned s2[2] = {0, 0};
         for (int wi = lane; wi < words; wi += 32) {
-            const int w = __ldg(xr + wi);
+            const int w = load_act(xr + wi);
             if (any[0]) {
                 s1[0] = __dp4a(w, 0x01010101, s1[0]);
                 s2[0] = (unsigned)__dp4a(w, w, (int)s2[0]);
@@ -484,7 +484,7 @@ analyze_layernorm_kernel(const int8_t* __restrict__ x, int64_t rows, int D, cons
             same[i] = i > 0 && i < n_cand && a.same_out[i] && F[i] == F[i - 1];
         double er[kAnMaxCand] = {0.0, 0.0, 0.0, 0.0};
         for (int wi = lane; wi < words; wi += 32) {
-            const unsigned w = (unsigned)__ldg(xr + wi);
+            const unsigned w = (unsigned)load_act(xr + wi);
             const unsigned sh = any[1] ? __ldg(reinterpret_cast<const unsigned*>(ptf) + wi) : 0u;
             // the four channels side by side under each uniform test: a row is one chain of fp64 latencies otherwise
             int xv[2][4];

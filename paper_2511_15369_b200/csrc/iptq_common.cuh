@@ -69,6 +69,34 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 // Allows the next kernel on the stream to be scheduled once every CTA of this grid has passed this point.
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Reads of an int8 / uint8 tensor, which the launch before may still be writing when this kernel starts (tables, weights,
+// indices and int32 inputs are no launch's outputs and may be read with __ldg()).  __ldg() promises the hardware data that does not change
+// while the kernel runs, and that holds only for what was complete when it started; a plain load behind grid_dep_wait() does not.
+__device__ __forceinline__ int load_act(const int* p)
+{
+    int v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int4 load_act(const int4* p)
+{
+    int4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int load_act(const int8_t* p)
+{
+    int v;
+    asm volatile("ld.global.s8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned load_act(const uint8_t* p)
+{
+    unsigned v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 #endif  // __CUDACC__
 
 // ---------------------------------------------------------------- device arithmetic

@@ -30,7 +30,7 @@ __device__ __forceinline__ int ln_load_word(const LnSource& s, int64_t row, int 
     for (int p = 1; p < 4; ++p)
         if (wi >= s.part_words) { wi -= s.part_words; ++part; }
     const int r = __ldg(s.index + row * s.parts + part);
-    return r < 0 ? 0 : __ldg(reinterpret_cast<const int*>(s.x) + (int64_t)r * s.part_words + wi);
+    return r < 0 ? 0 : load_act(reinterpret_cast<const int*>(s.x) + (int64_t)r * s.part_words + wi);
 }
 
 // ---- one row's constants.  n = ((D x - s1) F) >> 30 = hi32(v F) with v = 4 (D x - s1) and F up to 2^40: a high multiply by the

@@ -8,7 +8,7 @@
 namespace iptq {
 
 __global__ void __launch_bounds__(256)
-gather_rows_kernel(const int4* __restrict__ src, int4* __restrict__ dst, const int32_t* __restrict__ index,
+gather_rows_kernel(const int4* src, int4* __restrict__ dst, const int32_t* __restrict__ index,
                    int64_t n_dst, int parts, int vec_per_part)
 {
     grid_dep_launch();
@@ -22,7 +22,7 @@ gather_rows_kernel(const int4* __restrict__ src, int4* __restrict__ dst, const i
         const int part = v / vec_per_part;
         const int s = __ldg(index + row * parts + part);
         int4 val = make_int4(0, 0, 0, 0);
-        if (s >= 0) val = __ldg(src + (int64_t)s * vec_per_part + (v - part * vec_per_part));
+        if (s >= 0) val = load_act(src + (int64_t)s * vec_per_part + (v - part * vec_per_part));
         dst[i] = val;
     }
 }
@@ -30,7 +30,7 @@ gather_rows_kernel(const int4* __restrict__ src, int4* __restrict__ dst, const i
 // Image -> patch rows: out[(b, py, px), (c, dy, dx)] = img[b, c, py P + dy, px P + dx].  One 16-byte piece of a
 // patch line per thread per step; P is a multiple of 16, so every piece is aligned on both sides.
 __global__ void __launch_bounds__(256)
-patchify_kernel(const int4* __restrict__ img, int4* __restrict__ out, int64_t B, int C, int H, int W, int P)
+patchify_kernel(const int4* img, int4* __restrict__ out, int64_t B, int C, int H, int W, int P)
 {
     grid_dep_launch();
     grid_dep_wait();
@@ -48,7 +48,7 @@ patchify_kernel(const int4* __restrict__ img, int4* __restrict__ out, int64_t B,
         const int py = (int)((row / gw) % gh);
         const int64_t b = row / ((int64_t)gw * gh);
         const int64_t src = (((b * C + c) * H + (int64_t)py * P + dy) * W + (int64_t)px * P) / 16 + piece;
-        out[i] = __ldg(img + src);
+        out[i] = load_act(img + src);
     }
 }
 

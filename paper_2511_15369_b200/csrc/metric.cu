@@ -50,7 +50,7 @@ metric_finish_kernel(const double* __restrict__ work, int nblocks, double* __res
 
 // Softmax: a warp per row.  X_j = exp(z_j - z_max) / sum_k exp(z_k - z_max) with z = in_scale * score (fp64).
 __global__ void __launch_bounds__(kMetricThreads)
-metric_softmax_kernel(const int32_t* __restrict__ scores, const uint8_t* __restrict__ probs, int64_t rows, int n,
+metric_softmax_kernel(const int32_t* __restrict__ scores, const uint8_t* probs, int64_t rows, int n,
                       double in_scale, double out_step, double* __restrict__ work)
 {
     grid_dep_wait();
@@ -70,7 +70,7 @@ metric_softmax_kernel(const int32_t* __restrict__ scores, const uint8_t* __restr
         den = warp_sum(den);
         for (int j = lane; j < n; j += 32) {
             const double X = exp((double)__ldg(sr + j) * in_scale - zmax) / den;
-            const unsigned pb = __ldg(pr + j);
+            const unsigned pb = load_act(pr + j);
             // out_step = 0: the byte is a logarithm-candidate code, 2^-code (255: zero) built from the exponent bits
             const double Qd = out_step != 0.0 ? (double)pb * out_step
                                               : (pb == IPTQ_LOG2_ZERO ? 0.0 : __longlong_as_double((long long)(1023 - (int)min(pb, 15u)) << 52));
@@ -84,7 +84,7 @@ metric_softmax_kernel(const int32_t* __restrict__ scores, const uint8_t* __restr
 
 // GELU: element-wise.  X = v/2 (1 + erf(v / sqrt 2)), v = in_scale * x.
 __global__ void __launch_bounds__(kMetricThreads)
-metric_gelu_kernel(const int32_t* __restrict__ x, const int8_t* __restrict__ y, int64_t n, double in_scale,
+metric_gelu_kernel(const int32_t* __restrict__ x, const int8_t* y, int64_t n, double in_scale,
                    double out_scale, int out_zp, double* __restrict__ work)
 {
     grid_dep_wait();
@@ -93,7 +93,7 @@ metric_gelu_kernel(const int32_t* __restrict__ x, const int8_t* __restrict__ y, 
     for (int64_t i = (int64_t)blockIdx.x * kMetricThreads + threadIdx.x; i < n; i += stride) {
         const double v = (double)__ldg(x + i) * in_scale;
         const double X = 0.5 * v * (1.0 + erf(v / 1.4142135623730951));
-        const double d = X - (double)((int)__ldg(y + i) - out_zp) * out_scale;
+        const double d = X - (double)(load_act(y + i) - out_zp) * out_scale;
         ax2 += X * X;
         ae2 += d * d;
     }
@@ -102,7 +102,7 @@ metric_gelu_kernel(const int32_t* __restrict__ x, const int8_t* __restrict__ y, 
 
 // LayerNorm: a warp per row.  Mean from the exact integer sum, biased variance, no epsilon.
 __global__ void __launch_bounds__(kMetricThreads)
-metric_layernorm_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__ y, int64_t rows, int D,
+metric_layernorm_kernel(const int8_t* x, const int8_t* y, int64_t rows, int D,
                         const float* __restrict__ gamma, const float* __restrict__ beta,
                         const uint8_t* __restrict__ ptf, double out_scale, int out_zp, double* __restrict__ work)
 {
@@ -115,21 +115,21 @@ metric_layernorm_kernel(const int8_t* __restrict__ x, const int8_t* __restrict__
         const int8_t* xr = x + row * D;
         const int8_t* yr = y + row * D;
         long long s1 = 0;
-        for (int j = lane; j < D; j += 32) s1 += (long long)((int)xr[j] << (ptf ? (int)ptf[j] : 0));
+        for (int j = lane; j < D; j += 32) s1 += (long long)(load_act(xr + j) << (ptf ? (int)ptf[j] : 0));
 #pragma unroll
         for (int o = 16; o; o >>= 1) s1 += __shfl_xor_sync(kAll, s1, o);
         const double mu = (double)s1 / (double)D;
         double ss = 0.0;
         for (int j = lane; j < D; j += 32) {
-            const double c = (double)((int)xr[j] << (ptf ? (int)ptf[j] : 0)) - mu;
+            const double c = (double)(load_act(xr + j) << (ptf ? (int)ptf[j] : 0)) - mu;
             ss += c * c;
         }
         const double sd = sqrt(warp_sum(ss) / (double)D);
         for (int j = lane; j < D; j += 32) {
             const double b = (double)__ldg(beta + j);
             double X = b;
-            if (sd != 0.0) X = ((double)((int)xr[j] << (ptf ? (int)ptf[j] : 0)) - mu) / sd * (double)__ldg(gamma + j) + b;
-            const double d = X - (double)((int)yr[j] - out_zp) * out_scale;
+            if (sd != 0.0) X = ((double)(load_act(xr + j) << (ptf ? (int)ptf[j] : 0)) - mu) / sd * (double)__ldg(gamma + j) + b;
+            const double d = X - (double)(load_act(yr + j) - out_zp) * out_scale;
             ax2 += X * X;
             ae2 += d * d;
         }

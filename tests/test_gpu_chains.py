@@ -1,0 +1,53 @@
+"""Chains of dependent launches, run back to back many times: every launch may start while the one before it is still running,
+and each of these chains writes buffers that an earlier pass of it has read.  The last outputs have to be the first ones."""
+import numpy as np
+import pytest
+
+from paper_2511_15369_b200 import synth
+
+pytestmark = pytest.mark.gpu
+PASSES = 20
+
+
+@pytest.fixture(scope="module")
+def api():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2511_15369_b200 import api as _api
+    _api.lib()
+    return _api
+
+
+def _cu(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def test_gathers_and_patches_of_a_buffer_that_every_pass_rewrites(api):
+    """The readers of int8 activations that do not go through the copy engine, right behind the launch that writes them."""
+    import torch
+    g = np.random.default_rng(5)
+    src = [_cu(g.integers(-128, 128, size=(3136, 96)).astype(np.int8)) for _ in range(2)]
+    perm = _cu(g.permutation(3136).astype(np.int32).reshape(-1, 1))
+    four = _cu(g.integers(-1, 3136, size=(784, 4)).astype(np.int32))
+    gq, bq, c = api.layernorm_prepare(g.normal(1, 0.1, 384), g.normal(0, 0.1, 384), 8 / 127)
+    gq, bq = _cu(gq), _cu(bq)
+    buf, rows = torch.empty_like(src[0]), torch.empty((784, 384), dtype=torch.int8, device="cuda")
+
+    def one(x):
+        api.gather_rows(x, perm, out=buf)
+        n = api.layernorm_gather(buf, four, gq, bq, c)
+        api.gather_rows(buf, four, out=rows)
+        return n, api.layernorm(rows, gq, bq, c), api.patchify(buf.view(1, 3, 224, 448))
+    want = []
+    for x in src:
+        want.append(one(x))
+        torch.cuda.synchronize()
+    for i in range(PASSES):
+        got = [one(x) for x in src]
+    torch.cuda.synchronize()
+    for a, b in zip(want, got):
+        assert torch.equal(a[0], a[1])
+        assert all(torch.equal(p, q) for p, q in zip(a, b))
+    assert not torch.equal(want[0][0], want[1][0])

@@ -375,7 +375,8 @@ struct AnLayerNorm {
 };
 
 // The layer's parameters: by value in the launch up to MAXD channels (a copy to the device in front of every launch would
-// cost the stream more than a small layer's kernel), in device memory for wider layers.
+// cost the stream more than a small layer's kernel); for wider layers in the scratch, where launches that hold them by
+// value have put them (a copy from the caller's host memory would be recorded by a stream capture as a pointer to it).
 template <int MAXD>
 struct AnLnParams {
     float4 gamma[MAXD / 4], beta[MAXD / 4];
@@ -391,9 +392,33 @@ struct AnLnParams<0> {
     const int4 *gamma_q, *beta_q;
     __device__ __forceinline__ void get(int i, float4& g, float4& b, int4& gq, int4& bq) const
     {
-        g = __ldg(gamma + i); b = __ldg(beta + i); gq = __ldg(gamma_q + i); bq = __ldg(beta_q + i);
+        const int4 a = load_act(reinterpret_cast<const int4*>(gamma + i)), c = load_act(reinterpret_cast<const int4*>(beta + i));
+        g = make_float4(__int_as_float(a.x), __int_as_float(a.y), __int_as_float(a.z), __int_as_float(a.w));
+        b = make_float4(__int_as_float(c.x), __int_as_float(c.y), __int_as_float(c.z), __int_as_float(c.w));
+        gq = load_act(gamma_q + i); bq = load_act(beta_q + i);
     }
 };
+constexpr int kAnLnMaxDim = 3072;
+constexpr int kAnLnPart = 1536;                                          // channels per launch: 24 KB of parameters
+__global__ void __launch_bounds__(kAnThreads)
+analyze_layernorm_params_kernel(const __grid_constant__ AnLnParams<kAnLnPart> prm, int words, int first_word, int4* dst)
+{
+    grid_dep_launch();
+    const AnLnParams<kAnLnPart>* pp = &prm;                              // as in the kernel below
+    asm volatile("" : "+l"(pp));
+    grid_dep_wait();                                                     // an earlier launch may still be using this part of the scratch
+    const int i = blockIdx.x * kAnThreads + threadIdx.x;
+    if (i >= words) return;
+    float4 g, b;
+    int4 gq, bq;
+    pp->get(i, g, b, gq, bq);
+    int4* d = dst + first_word + i;
+    constexpr int W = kAnLnMaxDim / 4;
+    d[0] = make_int4(__float_as_int(g.x), __float_as_int(g.y), __float_as_int(g.z), __float_as_int(g.w));
+    d[W] = make_int4(__float_as_int(b.x), __float_as_int(b.y), __float_as_int(b.z), __float_as_int(b.w));
+    d[2 * W] = gq;
+    d[3 * W] = bq;
+}
 constexpr int kAnLnBytesPerChannel = 24;                                 // shared memory: two doubles, two ints
 
 // A warp per row, under two readings of its input: index 0 plain, 1 with the power-of-two factors.  The row is read twice (the
@@ -408,7 +433,7 @@ analyze_layernorm_kernel(const int8_t* x, int64_t rows, int D, const __grid_cons
     int2* gbq = reinterpret_cast<int2*>(gb + D);
     const int lane = threadIdx.x & 31, words = D >> 2;
     grid_dep_launch();
-    if (MAXD == 0) grid_dep_wait();                                      // the parameters were copied to the device just before
+    if (MAXD == 0) grid_dep_wait();                                      // the launches before this one write the parameters
     // Read through a generic pointer the compiler cannot trace back: as constant-bank loads with an address per lane these
     // reads go one address after the other, each a miss (10 us for 384 channels).
     const AnLnParams<MAXD>* pp = &prm;
@@ -644,7 +669,7 @@ int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* 
 {
     int rc = an_args_ok(consts, n_candidates, sums, work);
     if (rc != IPTQ_OK) return rc;
-    if (rows < 0 || dim < 4 || dim > 3072 || (dim & 3)) return IPTQ_ERR_SHAPE;
+    if (rows < 0 || dim < 4 || dim > kAnLnMaxDim || (dim & 3)) return IPTQ_ERR_SHAPE;
     if (!(out_scale > 0.0)) return IPTQ_ERR_SCALE_RANGE;
     if (!gamma || !beta || !gamma_q || !beta_q || (rows > 0 && !x)) return IPTQ_ERR_NULL;
     if (!aligned16(x) || (reinterpret_cast<uintptr_t>(ptf_shift) & 3u)) return IPTQ_ERR_ALIGN;
@@ -679,14 +704,19 @@ int iptq_analyze_layernorm(const int8_t* x, int64_t rows, int dim, const float* 
         AnLnParams<1024> prm;
         by_value(prm, analyze_layernorm_kernel<1024>);
     } else {
-        // where the GELU terms of another layer would be: the copies come after every earlier launch that uses the scratch
-        uint8_t* dst = static_cast<uint8_t*>(work) + kAnPartialBytes;
-        const void* src[4] = {gamma, beta, gamma_q, beta_q};
-        for (int i = 0; i < 4; ++i)
-            if (cudaMemcpyAsync(dst + (size_t)i * 3072 * 4, src[i], bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return IPTQ_ERR_CUDA;
-        AnLnParams<0> prm{reinterpret_cast<const float4*>(dst), reinterpret_cast<const float4*>(dst + 3072 * 4),
-                          reinterpret_cast<const int4*>(dst + 2 * 3072 * 4), reinterpret_cast<const int4*>(dst + 3 * 3072 * 4)};
-        if (cudaFuncSetAttribute(analyze_layernorm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnLnBytesPerChannel * 3072) != cudaSuccess)
+        // where the GELU terms of another layer would be
+        int4* dst = reinterpret_cast<int4*>(static_cast<uint8_t*>(work) + kAnPartialBytes);
+        for (int first = 0; first < dim; first += kAnLnPart) {
+            const int n = std::min(dim - first, kAnLnPart);
+            AnLnParams<kAnLnPart> part;
+            memcpy(part.gamma, gamma + first, (size_t)n * 4); memcpy(part.beta, beta + first, (size_t)n * 4);
+            memcpy(part.gamma_q, gamma_q + first, (size_t)n * 4); memcpy(part.beta_q, beta_q + first, (size_t)n * 4);
+            launch_kernel(analyze_layernorm_params_kernel, (n / 4 + kAnThreads - 1) / kAnThreads, kAnThreads, 0, stream, part, n / 4, first / 4, dst);
+            note_launch();
+        }
+        constexpr int W = kAnLnMaxDim / 4;
+        AnLnParams<0> prm{reinterpret_cast<const float4*>(dst), reinterpret_cast<const float4*>(dst + W), dst + 2 * W, dst + 3 * W};
+        if (cudaFuncSetAttribute(analyze_layernorm_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnLnBytesPerChannel * kAnLnMaxDim) != cudaSuccess)
             return IPTQ_ERR_CUDA;
         launch_kernel(analyze_layernorm_kernel<0>, grid, kAnThreads, smem, stream, x, rows, dim, prm, ptf_shift, out_scale, out_zp, a,
                       n_candidates, sums, counter, partials);

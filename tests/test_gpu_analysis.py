@@ -152,3 +152,25 @@ def test_codes_beyond_the_table(env, orc, n):
     X = metric.gelu_float(x, S)
     for c in layer.candidates:
         _same(c, metric.error_sums(X, metric.affine_deq(orc.gelu(x, orc.gelu_prepare(S, 16, So, zp, 8, c.variant)), So, zp)))
+
+
+@pytest.mark.parametrize("dim", [1028, 1536, 1540, 3072])
+def test_wide_layernorms_can_be_recorded(env, dim):
+    """A layer too wide for the launch's parameters, recorded into a graph and replayed after the caller's host arrays have changed."""
+    import torch
+    api, assign, metric = env
+    xf, gamma, beta, _ = synth.ln_values(20, dim, seed=dim)
+    x = _cu(synth.quantize_sym(xf, 8, np.int8)[0])
+    plain = assign.Analyzer()
+    plain.layernorm_layer("x", x, gamma, beta, 8.0 / 127, 3)
+    want = plain.finish()[0][0].candidates
+    an = assign.Analyzer()
+    graph, g, b = torch.cuda.CUDAGraph(), gamma.copy(), beta.copy()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        an.layernorm_layer("x", x, g, b, 8.0 / 127, 3)
+    g[:], b[:] = np.nan, np.nan
+    for _ in range(2):
+        graph.replay()
+    got = an.finish()[0][0].candidates
+    assert [(c.sum_x2, c.sum_err2) for c in got] == [(c.sum_x2, c.sum_err2) for c in want]

@@ -59,6 +59,7 @@ class Analyzer:
 
     def _add(self, layer, variants, launch, per_launch=api.ANALYZE_MAX_CANDIDATES):
         """Runs the candidates of one layer, as many per launch as a launch takes, and records them."""
+        variants = tuple(variants)
         for i in range(0, len(variants), per_launch):
             if self.n_eval >= self.max_evaluations:
                 raise RuntimeError("more evaluations than max_evaluations")

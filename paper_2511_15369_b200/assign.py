@@ -21,7 +21,7 @@ GELU_CANDIDATES = (api.GELU_POLY4, api.GELU_POLY2, api.GELU_SHIFT)
 LN_CANDIDATES = (api.LN_SHIFT, api.LN_NEWTON, api.LN_PTF)
 
 
-@dataclass(slots=True)
+@dataclass
 class Candidate:
     variant: int
     op_count: float
@@ -33,7 +33,7 @@ class Candidate:
     term: float = float("nan")
 
 
-@dataclass(slots=True)
+@dataclass
 class Layer:
     name: str
     kind: int

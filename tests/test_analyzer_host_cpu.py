@@ -25,3 +25,10 @@ def _analyzer(monkeypatch, launches, **kw):
 def test_candidates_from_any_iterable(monkeypatch, variants):
     an, layer = _analyzer(monkeypatch, _Launches())
     assert sorted(c.variant for c in layer(variants).candidates) == [0, 2]
+
+
+def test_results_take_attributes(monkeypatch):
+    an, layer = _analyzer(monkeypatch, _Launches())
+    l = layer((0,))
+    l.note = "kept"
+    l.candidates[0].note = "kept"

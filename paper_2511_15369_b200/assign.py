@@ -61,14 +61,13 @@ class Analyzer:
         """Runs the candidates of one layer, as many per launch as a launch takes, and records them."""
         variants = tuple(variants)
         for i in range(0, len(variants), per_launch):
-            if self.n_eval >= self.max_evaluations:
-                raise RuntimeError("more evaluations than max_evaluations")
+            # a launch that goes past the capacity writes its sums into the room behind it
             done = launch(variants[i:i + per_launch], self._sums_ptr + 16 * self.n_eval, self._work_ptr)
             for v, ops in done:
+                if self.n_eval >= self.max_evaluations:
+                    raise RuntimeError("more evaluations than max_evaluations")
                 layer.candidates.append(Candidate(v, ops, self.n_eval))
                 self.n_eval += 1
-            if self.n_eval > self.max_evaluations:
-                raise RuntimeError("more evaluations than max_evaluations")
         self.layers.append(layer)
         return layer
 

@@ -32,3 +32,18 @@ def test_results_take_attributes(monkeypatch):
     l = layer((0,))
     l.note = "kept"
     l.candidates[0].note = "kept"
+
+
+def test_the_capacity_counts_evaluations_alone(monkeypatch):
+    """Candidates without integer constants take no room, and a layer that does not fit leaves the layers before it as they are."""
+    ls = _Launches(applicable=(0, 1))
+    an, layer = _analyzer(monkeypatch, ls, max_evaluations=4)
+    assert [c.slot for c in layer((0, 1)).candidates] == [0, 1]
+    assert [c.slot for c in layer((0, 5, 1)).candidates] == [2, 3]
+    assert layer((5, 6)).candidates == []                      # full, and nothing to evaluate
+    for _ in range(3):
+        with pytest.raises(RuntimeError):
+            layer((0, 1))
+    assert len(an.layers) == 3 and an.n_eval == 4
+    room = an.sums.data_ptr() + 16 * an.sums.shape[0]
+    assert all(at + 16 * len(v) <= room for v, at in ls.seen)  # no launch can write past the buffer

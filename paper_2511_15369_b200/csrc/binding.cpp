@@ -116,6 +116,17 @@ void rank2(const at::Tensor& t)
     if (t.dim() != 2) fail(PyExc_ValueError, "expected a tensor of two dimensions");
 }
 cudaStream_t stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+// A library call without the interpreter's lock, which a launch into a full queue would otherwise keep from every other thread
+// until the device catches up.  The arguments have been read by then.
+template <typename... P, typename... A>
+int unlocked(int (*call)(P...), A... a)
+{
+    struct Unlock {
+        PyThreadState* state = PyEval_SaveThread();
+        ~Unlock() { PyEval_RestoreThread(state); }
+    } unlock;
+    return call(a...);
+}
 void check(int rc, const char* what)
 {
     if (rc == IPTQ_OK) return;
@@ -168,7 +179,7 @@ PyObject* softmax(PyObject* const* a, Py_ssize_t)
     rank2(x);
     const int64_t period = a[2] == Py_None ? 1 : tensor(a[2]).size(0);
     Out out(a[3], x.sizes(), at::kByte, x);
-    check(api.softmax(static_cast<const int32_t*>(x.data_ptr()), static_cast<uint8_t*>(out.ptr), x.size(0), (int)x.size(1),
+    check(unlocked(api.softmax, static_cast<const int32_t*>(x.data_ptr()), static_cast<uint8_t*>(out.ptr), x.size(0), (int)x.size(1),
                       dev<int32_t>(a[2]), period, host_struct<iptq_softmax_consts>(a[1]), stream()), "iptq_softmax");
     return out.result();
 }
@@ -178,7 +189,7 @@ PyObject* gelu(PyObject* const* a, Py_ssize_t)
 {
     const at::Tensor& x = device_tensor(a[0]);
     Out out(a[2], x.sizes(), at::kChar, x);
-    check(api.gelu(static_cast<const int32_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), x.numel(),
+    check(unlocked(api.gelu, static_cast<const int32_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), x.numel(),
                    host_struct<iptq_gelu_consts>(a[1]), stream()), "iptq_gelu");
     return out.result();
 }
@@ -189,7 +200,7 @@ PyObject* layernorm(PyObject* const* a, Py_ssize_t)
     const at::Tensor& x = device_tensor(a[0]);
     rank2(x);
     Out out(a[5], x.sizes(), at::kChar, x);
-    check(api.layernorm(static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), x.size(0), (int)x.size(1),
+    check(unlocked(api.layernorm, static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), x.size(0), (int)x.size(1),
                         dev<int32_t>(a[1]), dev<int32_t>(a[2]), dev<uint8_t>(a[4]), host_struct<iptq_ln_consts>(a[3]), stream()),
           "iptq_layernorm");
     return out.result();
@@ -203,7 +214,7 @@ PyObject* layernorm_gather(PyObject* const* a, Py_ssize_t)
     rank2(x); rank2(index);
     const int64_t rows = index.size(0), parts = index.size(1), sizes[2] = {rows, parts * x.size(1)};
     Out out(a[6], sizes, at::kChar, x);
-    check(api.layernorm_gather(static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), rows, (int)sizes[1],
+    check(unlocked(api.layernorm_gather, static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), rows, (int)sizes[1],
                                static_cast<const int32_t*>(index.data_ptr()), (int)parts, dev<int32_t>(a[2]), dev<int32_t>(a[3]),
                                dev<uint8_t>(a[5]), host_struct<iptq_ln_consts>(a[4]), stream()), "iptq_layernorm_gather");
     return out.result();
@@ -218,7 +229,7 @@ PyObject* linear(PyObject* const* a, Py_ssize_t)
     const int64_t M = x.size(0), K = x.size(1), N = w.size(0);
     const int64_t sizes[2] = {M, N};
     Out out(a[12], sizes, at::kChar, x);
-    check(api.linear_bits(static_cast<const int8_t*>(x.data_ptr()), w.data_ptr(), (int)integer(a[2]), dev<int32_t>(a[3]), dev<int32_t>(a[4]),
+    check(unlocked(api.linear_bits, static_cast<const int8_t*>(x.data_ptr()), w.data_ptr(), (int)integer(a[2]), dev<int32_t>(a[3]), dev<int32_t>(a[4]),
                           dev<int8_t>(a[5]), (int)integer(a[6]), dev<int8_t>(a[7]), host_struct<iptq_requant>(a[8]),
                           static_cast<int8_t*>(out.ptr), M, (int)N, (int)K, (int)integer(a[9]), address(a[10]),
                           (size_t)integer(a[11]), stream()), "iptq_linear");
@@ -233,7 +244,7 @@ PyObject* gather_rows(PyObject* const* a, Py_ssize_t)
     rank2(src); rank2(index);
     const int64_t sizes[2] = {index.size(0), index.size(1) * src.size(1)};
     Out out(a[2], sizes, at::kChar, src);
-    check(api.gather_rows(static_cast<const int8_t*>(src.data_ptr()), static_cast<int8_t*>(out.ptr),
+    check(unlocked(api.gather_rows, static_cast<const int8_t*>(src.data_ptr()), static_cast<int8_t*>(out.ptr),
                           static_cast<const int32_t*>(index.data_ptr()), index.size(0), (int)index.size(1), (int)src.size(1), stream()),
           "iptq_gather_rows");
     return out.result();
@@ -248,7 +259,7 @@ PyObject* patchify(PyObject* const* a, Py_ssize_t)
     const int64_t B = img.size(0), C = img.size(1), H = img.size(2), W = img.size(3);
     const int64_t sizes[2] = {B * (H / P) * (W / P), C * P * P};
     Out out(a[2], sizes, at::kChar, img);
-    check(api.patchify(static_cast<const int8_t*>(img.data_ptr()), static_cast<int8_t*>(out.ptr), B, (int)C, (int)H, (int)W, (int)P,
+    check(unlocked(api.patchify, static_cast<const int8_t*>(img.data_ptr()), static_cast<int8_t*>(out.ptr), B, (int)C, (int)H, (int)W, (int)P,
                        stream()), "iptq_patchify");
     return out.result();
 }
@@ -261,7 +272,7 @@ PyObject* attention_block(PyObject* const* a, Py_ssize_t)
     const int64_t B = q.size(0), H = q.size(1), N = q.size(2), dh = q.size(3);
     const int64_t sizes[3] = {B, N, H * dh};
     Out out(a[9], sizes, at::kChar, q);
-    check(api.attention_block(static_cast<const int8_t*>(q.data_ptr()), dev<int8_t>(a[1]), dev<int8_t>(a[2]), static_cast<int8_t*>(out.ptr),
+    check(unlocked(api.attention_block, static_cast<const int8_t*>(q.data_ptr()), dev<int8_t>(a[1]), dev<int8_t>(a[2]), static_cast<int8_t*>(out.ptr),
                               B, (int)H, (int)N, (int)dh, dev<int32_t>(a[7]), dev<int32_t>(a[10]), dev<uint8_t>(a[8]),
                               host_struct<iptq_softmax_consts>(a[3]), host_struct<iptq_requant>(a[4]), address(a[5]),
                               (size_t)integer(a[6]), stream()), "iptq_attention_block");
@@ -277,7 +288,7 @@ PyObject* mlp_block(PyObject* const* a, Py_ssize_t)
     const int64_t M = x.size(0), D = x.size(1), Dh = w1.size(0);
     const int64_t sizes[2] = {M, a[8] == Py_None ? Dh : D};
     Out out(a[16], sizes, at::kChar, x);
-    check(api.mlp_block(static_cast<const int8_t*>(x.data_ptr()), w1.data_ptr(), dev<int32_t>(a[2]), dev<int32_t>(a[3]), dev<int8_t>(a[4]),
+    check(unlocked(api.mlp_block, static_cast<const int8_t*>(x.data_ptr()), w1.data_ptr(), dev<int32_t>(a[2]), dev<int32_t>(a[3]), dev<int8_t>(a[4]),
                         host_struct<iptq_gelu_consts>(a[5]), dev<void>(a[8]), dev<int32_t>(a[9]), dev<int32_t>(a[10]),
                         dev<int8_t>(a[11]), (int)integer(a[12]), dev<int8_t>(a[13]), host_struct<iptq_requant>(a[14]),
                         static_cast<int8_t*>(out.ptr), M, (int)D, (int)Dh, (int)integer(a[15]), address(a[6]), (size_t)integer(a[7]),
@@ -291,7 +302,7 @@ PyObject* encoder_block(PyObject* const* a, Py_ssize_t)
     const at::Tensor& x = device_tensor(a[0]);
     rank2(x);
     Out out(a[1], x.sizes(), at::kChar, x);
-    check(api.encoder_block(static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), host_struct<iptq_block_params>(a[2]),
+    check(unlocked(api.encoder_block, static_cast<const int8_t*>(x.data_ptr()), static_cast<int8_t*>(out.ptr), host_struct<iptq_block_params>(a[2]),
                             address(a[3]), (size_t)integer(a[4]), stream()), "iptq_encoder_block");
     return out.result();
 }
@@ -339,7 +350,7 @@ PyObject* analyze_softmax(PyObject* const* a, Py_ssize_t)
         return api.softmax_prepare(scale, (int)x.size(1), v == IPTQ_SM_LOG2 ? 4 : bits, (iptq_softmax_variant)v, out);   // 4-bit codes
     });
     if (n)
-        check(api.analyze_softmax(static_cast<const int32_t*>(x.data_ptr()), x.size(0), (int)x.size(1), scale, c, n,
+        check(unlocked(api.analyze_softmax, static_cast<const int32_t*>(x.data_ptr()), x.size(0), (int)x.size(1), scale, c, n,
                                   static_cast<double*>(address(a[4])), address(a[5]), stream()), "iptq_analyze_softmax");
     return candidate_list(IPTQ_LAYER_SOFTMAX, ids, n, x.size(0), x.size(1));
 }
@@ -356,7 +367,7 @@ PyObject* analyze_gelu(PyObject* const* a, Py_ssize_t)
         return api.gelu_prepare(in_scale, in_bits, out_scale, zp, bits, (iptq_gelu_variant)v, out);
     });
     if (n)
-        check(api.analyze_gelu(static_cast<const int32_t*>(x.data_ptr()), x.numel(), in_scale, out_scale, zp, c, n,
+        check(unlocked(api.analyze_gelu, static_cast<const int32_t*>(x.data_ptr()), x.numel(), in_scale, out_scale, zp, c, n,
                                static_cast<double*>(address(a[7])), address(a[8]), stream()), "iptq_analyze_gelu");
     return candidate_list(IPTQ_LAYER_GELU, ids, n, x.numel(), 1);
 }
@@ -384,7 +395,7 @@ PyObject* analyze_layernorm(PyObject* const* a, Py_ssize_t)
         return (int)IPTQ_OK;
     });
     if (n)
-        check(api.analyze_layernorm(static_cast<const int8_t*>(x.data_ptr()), x.size(0), dim, gamma, beta, gq, bq, dev<uint8_t>(a[7]),
+        check(unlocked(api.analyze_layernorm, static_cast<const int8_t*>(x.data_ptr()), x.size(0), dim, gamma, beta, gq, bq, dev<uint8_t>(a[7]),
                                     out_scale, zp, c, n, static_cast<double*>(address(a[8])), address(a[9]), stream()),
               "iptq_analyze_layernorm");
     return candidate_list(IPTQ_LAYER_LAYERNORM, ids, n, x.size(0), dim);

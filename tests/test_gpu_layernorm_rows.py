@@ -46,3 +46,63 @@ def test_rows_and_widths(api, orc, variant, rows, dim):
         want = orc.layernorm(x, gq, bq, c, ptf)
         bad = np.argwhere(got != want)
         assert bad.size == 0, (len(bad), bad[:3].tolist())
+
+
+# the remaining kernels of the dispatch: one to four rows per warp at 52 .. 112, 384, 512, 1024 and 2048 channels, rows that fill their
+# words exactly and rows that do not
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("rows,dim", [(4740, 52), (18947, 80), (18946, 112), (4743, 384), (18945, 384), (18950, 260), (4738, 512), (18947, 512),
+                                      (18946, 388), (4737, 1024), (18945, 1024), (18946, 900), (4738, 2048), (4737, 1540)])
+def test_the_remaining_rows_per_warp(api, orc, variant, rows, dim):
+    test_rows_and_widths(api, orc, variant, rows, dim)
+
+
+def _general(api, orc, g, dim, variant):
+    """Parameters whose zero point does not fit into the rounding constant (outputs coarser than gamma); beta as large as its 32 bits allow."""
+    gamma = g.normal(0.2, 0.02, dim).astype(np.float32)
+    top = float(np.abs(gamma).max())
+    beta = (g.uniform(-1, 1, dim) * top * min(30.0, 0.9 * (64 - 1.125 * np.sqrt(dim)))).astype(np.float32)
+    for zp, out_scale in ((100, 2.05 * top), (-100, 3 * top), (-128, 9 * top), (0, 200 * top)):
+        gq, bq, c = orc.layernorm_prepare(gamma, beta, out_scale, zp, 8, variant)
+        _, _, ca = api.layernorm_prepare(gamma, beta, out_scale, zp, 8, variant)
+        assert abs((1 << (ca.out.shift - 1)) + (zp << ca.out.shift)) >= 1 << 30
+        yield gq, bq, c, ca
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("rows,dim", [(1, 4), (70, 96), (333, 128), (65, 200), (9, 3072)])
+def test_zero_points_beyond_the_rounding_constant(api, orc, variant, rows, dim):
+    import torch
+    g = np.random.default_rng(rows + dim)
+    x = _rows(g, rows, dim)
+    ptf = g.integers(0, 4, dim).astype(np.uint8) if variant == 2 else None
+    cu = lambda a: None if a is None else torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    kinds = 0
+    for gq, bq, c, ca in _general(api, orc, g, dim, variant):
+        want = orc.layernorm(x, gq, bq, c, ptf)
+        kinds = max(kinds, len(np.unique(want)))
+        assert (api.layernorm(cu(x), cu(gq), cu(bq), ca, cu(ptf)).cpu().numpy() == want).all()
+    assert kinds > (20 if dim in (96, 128, 200) else 3)
+
+
+@pytest.mark.parametrize("general", [False, True])
+@pytest.mark.parametrize("variant", [1, 2])
+@pytest.mark.parametrize("rows,C,parts", [(70, 96, 1), (5, 64, 1), (301, 48, 4), (4740, 96, 4), (19000, 24, 3), (90, 768, 4)])
+def test_gathered_rows_of_every_kind(api, orc, general, variant, rows, C, parts):
+    """Gathered LayerNorm with power-of-two factors, a zero point, and a zero point beyond the rounding constant."""
+    import torch
+    g = np.random.default_rng(rows + C)
+    x = _rows(g, 500, C)
+    idx = g.integers(-1, 500, size=(rows, parts)).astype(np.int32)
+    dim = C * parts
+    src = np.ascontiguousarray(np.where((idx >= 0)[:, :, None], x[np.maximum(idx, 0)], 0).reshape(rows, dim).astype(np.int8))
+    ptf = g.integers(0, 4, dim).astype(np.uint8) if variant == 2 else None
+    if general:
+        gq, bq, c, ca = next(_general(api, orc, g, dim, variant))
+    else:
+        gamma, beta = g.normal(1.0, 0.2, dim).astype(np.float32), g.normal(0.0, 0.2, dim).astype(np.float32)
+        gq, bq, c = orc.layernorm_prepare(gamma, beta, 8 / 127, -9, 8, variant)
+        _, _, ca = api.layernorm_prepare(gamma, beta, 8 / 127, -9, 8, variant)
+    cu = lambda a: None if a is None else torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    got = api.layernorm_gather(cu(x), cu(idx), cu(gq), cu(bq), ca, cu(ptf)).cpu().numpy()
+    assert (got == orc.layernorm(src, gq, bq, c, ptf)).all()

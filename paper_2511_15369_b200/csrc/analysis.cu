@@ -120,8 +120,8 @@ __device__ __forceinline__ double an_softmax_err(const AnSoftmaxCand& c, const i
 }
 
 // exp(-d S) of an integer distance d >= 0 as the product of two tabulated exponentials, exp(-(d >> k) 2^k S) exp(-(d mod 2^k) S):
-// two shared-memory reads and a multiply (half a unit in the last place more than exp() itself) instead of some fifty
-// fp64 instructions.  The tables cover d S < kAnExpRange, beyond which the exponential is below 1e-30 and counts as 0.
+// two shared-memory reads and a multiply instead of some fifty fp64 instructions.  Each argument is rounded to 2^-53 of at most 70, each
+// exp() is off by a unit in its last place and the product is rounded once more: below 2e-14 relative.  The tables cover d S < kAnExpRange, beyond which the exponential is below 1e-30 and counts as 0.
 constexpr double kAnExpRange = 70.0;
 constexpr int kAnExpMaxEntries = 4096;
 struct AnExp {

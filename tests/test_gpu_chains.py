@@ -51,3 +51,49 @@ def test_gathers_and_patches_of_a_buffer_that_every_pass_rewrites(api):
         assert torch.equal(a[0], a[1])
         assert all(torch.equal(p, q) for p, q in zip(a, b))
     assert not torch.equal(want[0][0], want[1][0])
+
+
+def _passes(api, run, check):
+    """run() PASSES times eagerly and PASSES times as a recorded graph; every pass's launches follow the last one's at once."""
+    import torch
+    first = run().clone()
+    torch.cuda.synchronize()
+    check()
+    for _ in range(PASSES):
+        last = run()
+    torch.cuda.synchronize()
+    assert torch.equal(first, last)
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        out = run()
+    for _ in range(PASSES):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(first, out)
+    check()
+    assert len(torch.unique(first)) > 30
+
+
+@pytest.mark.parametrize("table", [(0, 0, 0, 0), (3, 1, 2, 1)])
+@pytest.mark.parametrize("shape", [synth.BlockShape("DeiT-T b1", 1, 197, 192, 3, 64, 768), synth.BlockShape("DeiT-S b64", 64, 197, 384, 6, 64, 1536),
+                                   synth.BlockShape("50 tokens", 40, 50, 384, 6, 64, 1536)])
+def test_encoder_blocks(api, shape, table):
+    spec = synth.make_block(shape, seed=1, calib_images=1)
+    blk, x = api.EncoderBlock(spec, table), _cu(spec.x)
+    _passes(api, lambda: blk(x), blk.ws.check)
+
+
+def test_a_small_backbone(api):
+    from paper_2511_15369_b200 import swin
+    spec = synth.make_swin(1, [dict(dim=96, heads=3, depth=2, grid=(20, 31)), dict(dim=192, heads=6, depth=2, grid=(10, 16)),
+                               dict(dim=384, heads=12, depth=2, grid=(5, 8))], seed=3)
+    net, x = swin.SwinBackbone(spec), _cu(spec.x)
+    _passes(api, lambda: net(x), net.check)
+
+
+def test_a_whole_model(api):
+    from paper_2511_15369_b200 import vit
+    spec = synth.make_vit("DeiT-T", 2, 1)
+    model, image = vit.VitModel(spec), _cu(spec.image)
+    _passes(api, lambda: model(image), model.check)

@@ -74,6 +74,7 @@ constexpr int EPI_WARPS = 16;            // 4 TMEM lane quadrants x 4 token quar
 constexpr int GEMM_THREADS = 32 * (2 + EPI_WARPS);
 constexpr int ACC_COLS = 256;            // TMEM columns between the two accumulators
 constexpr uint32_t TMEM_COLS = 512;
+// A CTA asks for all of the SM's shared memory, so that no CTA of a neighbouring launch runs beside it.
 constexpr int SMEM_LIMIT = 227 * 1024;
 
 struct GemmParams {
@@ -701,6 +702,7 @@ static int gemm_plan(GemmParams& p, int64_t M, bool residual, bool table, int sm
             gemm_layout(q1, best_tn, pair, residual, table, kblocks, 1, &sb1)) epi_bufs = 2;
     }
     if (gemm_layout(p, best_tn, pair, residual, table, kblocks, epi_bufs, smem_bytes) < 2) return IPTQ_ERR_SHAPE;
+    *smem_bytes = SMEM_LIMIT;                                 // whatever the layout needs: nothing else shares the SM
     const int64_t n_tt = (M + p.TN - 1) / p.TN;
     if ((int64_t)p.n_ct * n_tt > (int64_t)1 << 30) return IPTQ_ERR_SHAPE;
     p.n_tt = (int)n_tt;

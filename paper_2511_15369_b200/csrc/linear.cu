@@ -74,7 +74,6 @@ constexpr int EPI_WARPS = 16;            // 4 TMEM lane quadrants x 4 token quar
 constexpr int GEMM_THREADS = 32 * (2 + EPI_WARPS);
 constexpr int ACC_COLS = 256;            // TMEM columns between the two accumulators
 constexpr uint32_t TMEM_COLS = 512;
-// A CTA asks for all of the SM's shared memory, so that no CTA of a neighbouring launch runs beside it.
 constexpr int SMEM_LIMIT = 227 * 1024;
 
 struct GemmParams {
@@ -139,73 +138,13 @@ __device__ __forceinline__ int tile_tokens(const GemmParams& p, int tt)
     return min(p.TN, (p.M - tt * p.TN + 31) & ~31);
 }
 
-// One warp's share of a tile: 32 channels (one per lane) x 16 NCH tokens, out of TMEM, through R and what follows it, into
-// the warp's staging block.  Straight-line code: tile width, output range and the place of the zero point are template
-// parameters, because the tests and reconvergence points they would otherwise put into every chunk of 16 tokens were
-// a third of the epilogue's instructions, and the epilogue is bound by the instructions it issues.
-// No load is in flight across the choice between the copies of this function; hand_back() is called once the last one
-// has completed.
-// ZP_AFTER: the output zero point is added behind the shift instead of being part of crnd.
-template <int EPI, int GELU_VARIANT, int NCH, bool SAT8, bool ZP_AFTER, typename HandBack>
-__device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t tacc, int cm, int cs, int cb,
-                                              int crnd, uint32_t res_lane, uint32_t tab_mid, uint32_t out_word,
-                                              unsigned sel1, unsigned sel2, HandBack&& hand_back)
-{
-    uint32_t acc[2][16];
-    tmem_ld16(tacc, acc[0]);
-#pragma unroll
-    for (int ch = 0; ch < NCH; ++ch) {
-        tmem_wait_ld();                                        // chunk ch is in registers
-        if (ch + 1 < NCH) tmem_ld16(tacc + (uint32_t)((ch + 1) * 16), acc[(ch + 1) & 1]);   // in flight during the arithmetic
-        else hand_back();
-        // Three passes over the chunk, so that the shared-memory reads (volatile, hence kept in program order with the
-        // stores) are issued back to back instead of one per stored byte.
-        int v[16], r[16];
-        if (EPI == EPI_RESIDUAL) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                asm volatile("ld.shared.s8 %0, [%1];" : "=r"(r[j]) : "r"(res_lane + (uint32_t)((ch * 16 + j) * 32)));
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(r[j]) : "r"(tab_mid + (uint32_t)(r[j] * 4)));
-        }
-        // R of the header: hi32((acc + bias) * mult) + rounding constant, shifted.  The bias add is written as
-        // add-then-max against INT_MIN: a plain add is moved to the multiplier's pipe by the assembler, which is the
-        // pipe this loop is short of.
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            v[j] = mad_hi(__viaddmax_s32((int)acc[ch & 1][j], cb, p.acc_floor), cm, crnd) >> cs;
-            if (ZP_AFTER) v[j] += p.out_zp;
-            if (EPI == EPI_GELU_TAB) v[j] = max(-32768, min(32767, v[j])) + (int)tab_mid;
-            if (EPI == EPI_GELU) v[j] = requant_nosat(gelu_core<GELU_VARIANT>(v[j], p.gelu), p.gelu.out);
-            if (EPI == EPI_RESIDUAL) v[j] += r[j];
-            if (!SAT8) v[j] = EPI == EPI_GELU ? max(p.gelu.out.qmin, min(p.gelu.out.qmax, v[j])) : max(p.qmin, min(p.qmax, v[j]));
-        }
-        if (EPI == EPI_GELU_TAB) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v[j]) : "r"((uint32_t)v[j]));
-        }
-        // Four tokens of this lane's channel are packed into a word (saturating to int8), then a 4 x 4 byte transpose over
-        // the four lanes of a group (two shuffle + byte-permute rounds) leaves lane m of the group with token m of the
-        // four for the group's four channels: one 32-bit store per four outputs, every lane of the warp on its own bank
-        // (byte stores of four lanes into one word took 2.7 shared-memory passes each).
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            unsigned w = pack4_sat_s8(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-            w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), sel1);
-            w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 2), sel2);
-            asm volatile("st.shared.b32 [%0], %1;" ::"r"(out_word + (uint32_t)((ch * 16 + 4 * g) * 32)), "r"(w) : "memory");
-        }
-    }
-}
-
 // PAIR: two CTAs of a cluster compute 256 channels x TN tokens with one MMA stream (cta_group::2).  Each stages its
 // own 128 weight rows and HALF of the activation tile (TN / 2 tokens), which lowers the operand traffic per SM from
 // (128 + TN) to (128 + TN / 2) rows per 128-byte block of K; each receives its 128 channels x TN tokens in its own
 // TMEM, so the epilogue is the same as without pairs.  The even CTA issues the MMAs: its `full` barriers count the
 // bytes of both CTAs' copies, its `acc_empty` barriers the epilogue warps of both, and its commits signal the
 // `empty` and `acc_full` barriers of both.
-template <int EPI, int GELU_VARIANT, bool PAIR, int NCH>
+template <int EPI, int GELU_VARIANT, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
                const __grid_constant__ CUtensorMap map_y, const __grid_constant__ CUtensorMap map_res,
@@ -222,7 +161,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_bar + 2 * EPI_WARPS);
     CtaControl* ctl = reinterpret_cast<CtaControl*>(tmem_slot + 1);
 
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // the same in all lanes, and known to be
+    const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int kblocks = (p.K + BK - 1) / BK;
     const int stages = p.stages;
@@ -330,7 +269,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         const int ew = warp - 2;
         const int quad = warp & 3;
         const int part = ew >> 2;
-        constexpr int tpp = 16 * NCH;                          // tokens per part (TN / 4)
+        const int tpp = p.TN >> 2;                             // tokens per part: 16, 32, 48 or 64
+        const int nchunks = tpp >> 4;                          // 16-token chunks: 1..4
         // Staging blocks of this warp, [tpp tokens][32 channels] int8 each: one for the outputs and one for the
         // residual, or two of each used by alternate tiles.  With two, a tile neither waits for the copy engine to
         // have read the previous tile's outputs nor for a residual block that could only be requested once the
@@ -354,14 +294,14 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             for (int i = ew * 32 + lane; i < IPTQ_GELU_TABLE_SIZE / 16; i += EPI_WARPS * 32) dst[i] = __ldg(src + i);
             named_barrier(1, EPI_WARPS * 32);
         }
-        // The residual term R_res((res - zp) << 16) + out_zp depends on the residual byte alone: its 256 values are tabulated
+        // The residual term R_res((res - zp) << 16) depends on the residual byte alone: its 256 values are tabulated
         // once per CTA, with the arithmetic the epilogue would otherwise run per output, and an output then costs a
         // second shared-memory read instead of a high multiply and a shift.
         const uint32_t rlut_mid = smem_u32(smem + p.off_tab) + 512u;        // address of the entry of residual byte 0
         if (EPI == EPI_RESIDUAL) {
             int* rl = reinterpret_cast<int*>(smem + p.off_tab);
             const int i = ew * 32 + lane;
-            if (i < 256) rl[i] = requant_core((i - 128) * 65536 - p.res_off, p.res_mult, p.res_rnd, p.res_shift) + p.out_zp;
+            if (i < 256) rl[i] = requant_core((i - 128) * 65536 - p.res_off, p.res_mult, p.res_rnd, p.res_shift);
             named_barrier(1, EPI_WARPS * 32);
         }
         grid_dep_wait();                                       // residual reads and output writes come after this
@@ -409,44 +349,103 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
             const int tok0 = tt * p.TN + part * tpp;          // first token of this warp
             const bool active = c0 < p.N && tok0 < p.M;       // warp-uniform
             // The output zero point, which is added after the shift, goes into the rounding constant, shifted left,
-            // where every channel of the warp has a shift small enough for that (the sum stays below 2^31).  The residual
-            // epilogue has it in the table of residual terms, the GELU epilogues have none.
-            const bool fold = EPI != EPI_REQUANT || __all_sync(0xffffffffu, cs <= 20);
-            const int crnd = (1 << (cs - 1)) + (EPI == EPI_REQUANT && fold ? p.out_zp << cs : 0);
+            // where every channel of the warp has a shift small enough for that (the sum stays below 2^31).
+            const bool fold = EPI == EPI_REQUANT && __all_sync(0xffffffffu, cs <= 20);
+            const int crnd = (1 << (cs - 1)) + (fold ? p.out_zp << cs : 0);
+            // the residual epilogue, whose other half already is an add and a high multiply per output, is faster with
+            // bias and rounding constant in the 64-bit addend of one wide multiply-add (measured: 5 % at K = 96)
+            const long long c64 = (long long)cb * (long long)cm + ((long long)(1 << (cs - 1)) << 32);
             if (!mbar_wait_warp(&acc_full[ab], abph, ctl, p.status, 4)) break;
             tc_fence_after_sync();
+            // the store that last used this tile's output block has read it (one or two K loops ago)
+            if (lane == 0) { if (two) bulk_wait_read_but_one(); else bulk_wait_read_all(); }
+            __syncwarp();
+            if (EPI == EPI_RESIDUAL && active) {
+                if (!mbar_wait_warp(&res_bar[2 * ew + sb], (res_ph >> sb) & 1u, ctl, p.status, 5)) break;
+                res_ph ^= 1u << sb;
+            }
             const uint32_t tacc = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ab * ACC_COLS + part * tpp);
-            auto hand_back = [&] {                             // the MMA warp may refill this accumulator
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) {
-                    if (PAIR) mbar_arrive_cluster(acc_empty0 + (uint32_t)(ab * 8)); else mbar_arrive(&acc_empty[ab]);
+            uint32_t acc[2][16];
+            tmem_ld16(tacc, acc[0]);
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {
+                if (ch < nchunks) {                            // warp-uniform
+                    tmem_wait_ld();                            // chunk ch is in registers
+                    if (ch + 1 < nchunks) {
+                        tmem_ld16(tacc + (uint32_t)((ch + 1) * 16), acc[(ch + 1) & 1]);   // in flight during the arithmetic
+                    } else {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) {                       // the MMA warp may refill this accumulator
+                            if (PAIR) mbar_arrive_cluster(acc_empty0 + (uint32_t)(ab * 8)); else mbar_arrive(&acc_empty[ab]);
+                        }
+                    }
+                    if (active) {
+                        // Three passes over the chunk, so that the shared-memory reads (volatile, hence kept in
+                        // program order with the stores) are issued back to back instead of one per stored byte.
+                        int v[16], r[16];
+                        if (EPI == EPI_RESIDUAL) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                asm volatile("ld.shared.s8 %0, [%1];" : "=r"(r[j]) : "r"(res_lane + (uint32_t)((ch * 16 + j) * 32)));
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(r[j]) : "r"(rlut_mid + (uint32_t)(r[j] * 4)));
+                        }
+                        // R of the header: hi32((acc + bias) * mult) + rounding constant, shifted.  The bias add is
+                        // written as add-then-max against INT_MIN: a plain add is moved to the multiplier's pipe by the
+                        // assembler, which is the pipe this loop is short of.
+                        if (fold) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                v[j] = mad_hi(__viaddmax_s32((int)acc[ch & 1][j], cb, p.acc_floor), cm, crnd) >> cs;
+                                if (!sat8) v[j] = max(p.qmin, min(p.qmax, v[j]));
+                            }
+                        } else
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            if (EPI == EPI_RESIDUAL) v[j] = mad_wide_hi((int)acc[ch & 1][j], cm, c64) >> cs;
+                            else v[j] = mad_hi(__viaddmax_s32((int)acc[ch & 1][j], cb, p.acc_floor), cm, crnd) >> cs;
+                            if (EPI == EPI_GELU_TAB) {
+                                v[j] = max(-32768, min(32767, v[j])) + (int)tab_mid;
+                            } else if (EPI == EPI_GELU) {
+                                v[j] = requant_nosat(gelu_core<GELU_VARIANT>(v[j], p.gelu), p.gelu.out);
+                                if (!sat8) v[j] = max(p.gelu.out.qmin, min(p.gelu.out.qmax, v[j]));
+                            } else if (EPI == EPI_RESIDUAL) {
+                                v[j] += r[j] + p.out_zp;
+                                if (!sat8) v[j] = max(p.qmin, min(p.qmax, v[j]));
+                            } else {
+                                v[j] += p.out_zp;
+                                if (!sat8) v[j] = max(p.qmin, min(p.qmax, v[j]));
+                            }
+                        }
+                        if (EPI == EPI_GELU_TAB) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j)
+                                asm volatile("ld.shared.s8 %0, [%1];" : "=r"(v[j]) : "r"((uint32_t)v[j]));
+                        }
+                        // Four tokens of this lane's channel are packed into a word (saturating to int8), then a 4 x 4
+                        // byte transpose over the four lanes of a group (two shuffle + byte-permute rounds) leaves
+                        // lane m of the group with token m of the four for the group's four channels: one 32-bit
+                        // store per four outputs, every lane of the warp on its own bank (byte stores of four lanes
+                        // into one word took 2.7 shared-memory passes each).
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            unsigned w = pack4_sat_s8(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+                            w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), sel1);
+                            w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 2), sel2);
+                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(out_word + (uint32_t)((ch * 16 + 4 * g) * 32)), "r"(w) : "memory");
+                        }
+                    }
                 }
-            };
+            }
             if (active) {
-                // the store that last used this tile's output block has read it (one or two K loops ago)
-                if (lane == 0) { if (two) bulk_wait_read_but_one(); else bulk_wait_read_all(); }
-                __syncwarp();
-                if (EPI == EPI_RESIDUAL) {
-                    if (!mbar_wait_warp(&res_bar[2 * ew + sb], (res_ph >> sb) & 1u, ctl, p.status, 5)) break;
-                    res_ph ^= 1u << sb;
-                }
-                const uint32_t tab = EPI == EPI_RESIDUAL ? rlut_mid : tab_mid;
-                if (!fold)
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, true>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
-                else if (EPI == EPI_GELU_TAB || sat8)
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, true, false>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
-                else
-                    epilogue_tile<EPI, GELU_VARIANT, NCH, false, false>(p, tacc, cm, cs, cb, crnd, res_lane, tab, out_word, sel1, sel2, hand_back);
                 fence_proxy_async_smem();                     // this lane's shared-memory stores -> visible to the TMA engine
                 __syncwarp();
                 if (lane == 0) {
                     tma_store_2d(&map_y, out_blk0 + (uint32_t)sb * buf_bytes, c0, tok0);  // clipped at N and M
                     bulk_commit();
                 }
-            } else {
-                hand_back();
-                if (lane == 0) bulk_commit();                  // an empty group: the wait above counts one group per tile
             }
             __syncwarp();                                      // every lane has read its residual bytes of this tile
             if (EPI == EPI_RESIDUAL && !two && nhave) request_residual(ntt, nct, 0);
@@ -568,11 +567,11 @@ int unpack_int4_launch(const void* packed, int8_t* out, int64_t n_elems, cudaStr
 }
 
 // ---------------------------------------------------------------- launcher
-template <int EPI, int GV, bool PAIR, int NCH>
+template <int EPI, int GV, bool PAIR>
 static int launch_gemm_as(const CUtensorMap& mw, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mr,
                           const GemmParams& p, int grid, int smem_bytes, cudaStream_t st)
 {
-    auto kern = gemm_i8_kernel<EPI, GV, PAIR, NCH>;
+    auto kern = gemm_i8_kernel<EPI, GV, PAIR>;
     static bool configured[64];               // one attribute call per instantiation and device
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return IPTQ_ERR_CUDA;
@@ -591,15 +590,8 @@ template <int EPI, int GV>
 static int launch_gemm(const CUtensorMap& mw, const CUtensorMap& mx, const CUtensorMap& my, const CUtensorMap& mr,
                        const GemmParams& p, bool pair, int grid, int smem_bytes, cudaStream_t st)
 {
-    if (pair) return launch_gemm_as<EPI, GV, true, 4>(mw, mx, my, mr, p, grid, smem_bytes, st);   // pairs take 256-token tiles
-    switch (p.TN) {
-        case 64: return launch_gemm_as<EPI, GV, false, 1>(mw, mx, my, mr, p, grid, smem_bytes, st);
-        case 128: return launch_gemm_as<EPI, GV, false, 2>(mw, mx, my, mr, p, grid, smem_bytes, st);
-        case 192:
-            if constexpr (EPI == EPI_GELU_TAB) return launch_gemm_as<EPI, GV, false, 3>(mw, mx, my, mr, p, grid, smem_bytes, st);
-            else return IPTQ_ERR_SHAPE;                       // never planned
-        default: return launch_gemm_as<EPI, GV, false, 4>(mw, mx, my, mr, p, grid, smem_bytes, st);
-    }
+    return pair ? launch_gemm_as<EPI, GV, true>(mw, mx, my, mr, p, grid, smem_bytes, st)
+                : launch_gemm_as<EPI, GV, false>(mw, mx, my, mr, p, grid, smem_bytes, st);
 }
 
 int linear_check(const LinearArgs& a)
@@ -686,7 +678,7 @@ static int gemm_plan(GemmParams& p, int64_t M, bool residual, bool table, int sm
         GemmParams q = p;
         int sb;
         if (TN > 64 && M <= TN - 64) continue;                // a narrower tile covers all tokens
-        if (TN == 192 && !table) continue;                    // that width stands in for 256 beside the GELU table, and is built for it alone
+        if (TN == 192 && !table) continue;                    // that width stands in for 256 beside the GELU table
         if (gemm_layout(q, TN, false, residual, table, kblocks, 1, &sb) < std::min(3, kblocks + 1)) continue;
         best_tn = TN;
         break;
@@ -702,7 +694,6 @@ static int gemm_plan(GemmParams& p, int64_t M, bool residual, bool table, int sm
             gemm_layout(q1, best_tn, pair, residual, table, kblocks, 1, &sb1)) epi_bufs = 2;
     }
     if (gemm_layout(p, best_tn, pair, residual, table, kblocks, epi_bufs, smem_bytes) < 2) return IPTQ_ERR_SHAPE;
-    *smem_bytes = SMEM_LIMIT;                                 // whatever the layout needs: nothing else shares the SM
     const int64_t n_tt = (M + p.TN - 1) / p.TN;
     if ((int64_t)p.n_ct * n_tt > (int64_t)1 << 30) return IPTQ_ERR_SHAPE;
     p.n_tt = (int)n_tt;

@@ -120,8 +120,8 @@ __device__ __forceinline__ bool mbar_wait_nocall(uint64_t* bar, uint32_t parity,
 
 // The same wait for a whole warp.  A barrier that completes between the lanes' tries splits the warp, and what follows these
 // waits (TMEM loads, named barriers) is .aligned: the vote joins the lanes again and they all go the same way.  One lane
-// polling for all, with a shuffle behind it, does so too, but costs a round trip more per wait: every pass of the encoder
-// block was 2 to 9 % slower (DeiT-Tiny batch 1 29.7 us, 27.0 with the vote; ViT-Base batch 128 291.8, 287.0).
+// polling for all, with a shuffle behind it, does so too, but costs a round trip more per wait (ViT-Base block at batch 128
+// 291.8 us, 287.0 with the vote; a DeiT-Tiny block of one image 29.7, 27.0).
 template <bool CALL = true>
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, CtaControl* ctl, StatusBlock* status, int where)
 {

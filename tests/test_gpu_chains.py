@@ -97,3 +97,35 @@ def test_a_whole_model(api):
     spec = synth.make_vit("DeiT-T", 2, 1)
     model, image = vit.VitModel(spec), _cu(spec.image)
     _passes(api, lambda: model(image), model.check)
+
+
+@pytest.mark.parametrize("table", [(0, 0, 0, 0), (3, 1, 2, 1)])
+def test_fresh_states(api, table):
+    """First passes of one block state after the other, each in memory of its own that goes back to the device in between: every first pass and
+    every replay gives the same bytes, and nothing reaches for memory that is no longer there."""
+    import gc
+
+    import torch
+    spec = synth.make_block(synth.BlockShape("DeiT-S b64", 64, 197, 384, 6, 64, 1536), seed=1, calib_images=1)
+    rng, want = np.random.default_rng(0), None
+    for n in range(60):
+        pad = torch.empty(int(rng.integers(1, 40)) << 20, dtype=torch.uint8, device="cuda")
+        blk, x = api.EncoderBlock(spec, table), _cu(spec.x)
+        torch.cuda.synchronize()
+        y = blk(x)
+        torch.cuda.synchronize()
+        got = y.cpu()
+        want = got if want is None else want
+        assert torch.equal(got, want), n
+        if n % 3 == 0:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                out = blk(x)
+            for _ in range(5):
+                graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, y), n
+            del graph, out
+        del pad, blk, x, y
+        gc.collect()
+        torch.cuda.empty_cache()
